@@ -101,16 +101,12 @@ struct AdjW {
 __device__ __forceinline__ AdjW make_adj_w(const Coef &c) {
   AdjW a;
   a.w = make_w(c, 0.0);
-  const double d[4] = {c.wx, c.wy, c.wz, c.wc};
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
-    a.wh[i] = __double2float_rn(d[i]);
-    a.wl[i] = __double2float_rn(__dsub_rn(d[i], (double)a.wh[i]));
+    a.wh[i] = c.wh[i];
+    a.wl[i] = c.wl[i];
   }
-  bool ok = true;
-#pragma unroll
-  for (int i = 0; i < 3; ++i) ok = ok && d[i] >= 0x1p-18 && d[i] <= 0x1p18;
-  a.pair = ok;
+  a.pair = c.pair != 0;
   return a;
 }
 

@@ -73,20 +73,19 @@ __device__ __forceinline__ W<double> make_w(const Coef &c, double) {
   w.wy = c.wy;
   w.wz = c.wz;
   w.wc = c.wc;
-  const double d[3] = {c.wx, c.wy, c.wz};
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
-    w.wh[i] = __double2float_rn(d[i]);
-    w.wl[i] = __double2float_rn(__dsub_rn(d[i], (double)w.wh[i]));
-    w.ah[i] = __fmul_rn(w.wh[i], 8388608.0f);
-    w.al[i] = __fmul_rn(w.wl[i], 8388608.0f);
+    w.wh[i] = c.wh[i];
+    w.wl[i] = c.wl[i];
+    w.ah[i] = c.ah[i];
+    w.al[i] = c.al[i];
   }
   w.emu = c.f64_emu != 0;
   w.ng = weight_groups(c.wx, c.wy, c.wz);
   return w;
 }
 __device__ __forceinline__ W<float> make_w(const Coef &c, float) {
-  return {(float)c.wx, (float)c.wy, (float)c.wz, (float)c.wc};
+  return {c.wh[0], c.wh[1], c.wh[2], c.wh[3]};
 }
 
 // The FP64 update of one inner point (see the file comment for the order).

@@ -27,6 +27,7 @@
 // including 2-D and 1-D ones: absent dimensions have zero neighbour strides
 // and zero weights).
 #include <algorithm>
+#include <cmath>
 #include <cstdint>
 #include <cstring>
 #include <mutex>
@@ -46,36 +47,37 @@ constexpr unsigned kGpWE = 40, kGpQE = 36;
 static_assert(kGpWE <= kPairMaxRadius && kGpQE <= kPairMaxRadius,
               "pair_ok radii must stay inside pair_split's range");
 
-// weights as pairs, the sign of the half step applied (x, y, z, centre);
-// dt and g as pairs
+// A half step's weights as pairs, its sign applied (x, y, z, centre), dt and g
+// as pairs, and the FP32 kernels' weights (kf: kx, ky, kz, kc without the
+// sign), all formed on the host (see Coef).
 struct GpPairW {
   double k[4];  // s kx, s ky, s kz, s kc (FP64)
-  float kh[4], kl[4];
+  float kh[4], kl[4], kf[4];
   double dt, g;
   float dth, dtl, gh, gl;
   float s;
-  bool pair;
+  int pair;
 };
 
-__device__ __forceinline__ GpPairW make_gp_w(const GpCoef &c, int which) {
+GpPairW make_gp_w(const GpCoef &c, int which) {
   GpPairW w;
   const double sg = which == 0 ? 1.0 : -1.0;
   const double d[4] = {c.kx, c.ky, c.kz, c.kc};
   bool ok = true;
-#pragma unroll
   for (int i = 0; i < 4; ++i) {
     w.k[i] = sg * d[i];
-    w.kh[i] = __double2float_rn(w.k[i]);
-    w.kl[i] = __double2float_rn(__dsub_rn(w.k[i], (double)w.kh[i]));
+    w.kh[i] = (float)w.k[i];
+    w.kl[i] = (float)(w.k[i] - (double)w.kh[i]);
+    w.kf[i] = (float)d[i];
     // (a zero weight: an absent dimension)
     if (i < 3) ok = ok && (d[i] == 0.0 || (fabs(d[i]) >= 0x1p-18 && fabs(d[i]) <= 0x1p18));
   }
   w.dt = c.dt;
   w.g = c.g;
-  w.dth = __double2float_rn(c.dt);
-  w.dtl = __double2float_rn(__dsub_rn(c.dt, (double)w.dth));
-  w.gh = __double2float_rn(c.g);
-  w.gl = __double2float_rn(__dsub_rn(c.g, (double)w.gh));
+  w.dth = (float)c.dt;
+  w.dtl = (float)(c.dt - (double)w.dth);
+  w.gh = (float)c.g;
+  w.gl = (float)(c.g - (double)w.gh);
   w.s = (float)sg;
   // dt and g enter the pair products: dt in [2^-40, 2^20], g zero or in
   // [2^-40, 2^40]
@@ -171,13 +173,12 @@ __device__ __forceinline__ double gp_out_f64(double o, double q, double wc, doub
 // o + s h for FP32 fields
 __device__ __forceinline__ float gp_out_f32(float o, float uc, float vc, float pot, float wc,
                                             float wxm, float wxp, float wym, float wyp, float wzm,
-                                            float wzp, const GpCoef &c, int which) {
-  const float kx = (float)c.kx, ky = (float)c.ky, kz = (float)c.kz, kc = (float)c.kc;
-  float h = __fmul_rn(kc, wc);
-  h = __fmaf_rn(kx, __fadd_rn(wxm, wxp), h);
-  h = __fmaf_rn(ky, __fadd_rn(wym, wyp), h);
-  h = __fmaf_rn(kz, __fadd_rn(wzm, wzp), h);
-  const float q = __fmul_rn((float)c.dt, __fmaf_rn((float)c.g, __fmaf_rn(uc, uc, __fmul_rn(vc, vc)), pot));
+                                            float wzp, const GpPairW &w, int which) {
+  float h = __fmul_rn(w.kf[3], wc);
+  h = __fmaf_rn(w.kf[0], __fadd_rn(wxm, wxp), h);
+  h = __fmaf_rn(w.kf[1], __fadd_rn(wym, wyp), h);
+  h = __fmaf_rn(w.kf[2], __fadd_rn(wzm, wzp), h);
+  const float q = __fmul_rn(w.dth, __fmaf_rn(w.gh, __fmaf_rn(uc, uc, __fmul_rn(vc, vc)), pot));
   h = __fmaf_rn(q, wc, h);
   return which == 0 ? __fadd_rn(o, h) : __fadd_rn(o, -h);
 }
@@ -192,7 +193,7 @@ constexpr int kGpX = 32, kGpY = 8, kGpZ = 32;
 template <class S, int WHICH>
 __global__ void __launch_bounds__(kGpX *kGpY)
     k_gp_half(int nx, int ny, int nz, int zchunks, S *__restrict__ u, S *__restrict__ v,
-              const S *__restrict__ V, GpCoef c) {
+              const S *__restrict__ V, const GpPairW pw) {
   const int ylo = ny > 1 ? 1 : 0, yhi = ny > 1 ? ny - 1 : 1;
   const int zlo = nz > 1 ? 1 : 0, zhi = nz > 1 ? nz - 1 : 1;
   const int i = 1 + blockIdx.x * kGpX + threadIdx.x, j = ylo + blockIdx.y * kGpY + threadIdx.y;
@@ -210,7 +211,6 @@ __global__ void __launch_bounds__(kGpX *kGpY)
   const S *Vs = V + sub * nloc;
   long long p = ii + (long long)nx * jj + (long long)nx * ny * k0;
   if constexpr (sizeof(S) == 8) {
-    const GpPairW pw = make_gp_w(c, WHICH);
     double wm = w[p - sz], wc = w[p];
     for (int k = k0; k < k1; ++k, p += (long long)nx * ny) {
       const double wp = w[p + sz];
@@ -238,7 +238,7 @@ __global__ void __launch_bounds__(kGpX *kGpY)
       const S o = out[p];
       const S uc = WHICH == 0 ? o : wc, vc = WHICH == 0 ? wc : o;
       const S r = gp_out_f32(o, uc, vc, Vs[p], wc, w[p - 1], w[p + 1], w[p - sy], w[p + sy], wm,
-                             wp, c, WHICH);
+                             wp, pw, WHICH);
       if (act) out[p] = r;
       wm = wc;
       wc = wp;
@@ -283,7 +283,8 @@ template <class S, int WHICH>
 __global__ void __launch_bounds__(32 * GpShape<S>::WARPS, 1)
     k_gp_tma(const __grid_constant__ CUtensorMap mW, const __grid_constant__ CUtensorMap mO,
              const __grid_constant__ CUtensorMap mV, int nx, int ny, int nz, int ncx, int ncxy,
-             int ncol, S *__restrict__ out, GpCoef c, unsigned *__restrict__ dev_err) {
+             int ncol, S *__restrict__ out, const GpPairW pw, const int *__restrict__ nbr, int ox,
+             int xsend, unsigned *__restrict__ dev_err) {
   using Sh = GpShape<S>;
   constexpr int V = Sh::V, W = Sh::W, BW = Sh::BW, H = Sh::H, NS = Sh::NS;
   constexpr unsigned NT = 32 * Sh::WARPS;
@@ -340,7 +341,6 @@ __global__ void __launch_bounds__(32 * GpShape<S>::WARPS, 1)
   }
   __syncthreads();
 
-  const GpPairW pw = make_gp_w(c, WHICH);
   const int r = warp;
   const int ob = (r + 1) * BW + V + lane * V;  // own points in the w box / pair plane
   const int oo = r * W + lane * V;             // own points in the o and V boxes
@@ -372,16 +372,16 @@ __global__ void __launch_bounds__(32 * GpShape<S>::WARPS, 1)
     // element offsets of their copies
     unsigned sendm = 0u;
     long long dr = 0, dl = 0;
-    if (c.xsend) {
-      const int sub = zoff / nz, xl = c.nbr[6 * sub], xr = c.nbr[6 * sub + 1];
-      const long long nloc = sz * nz, h = nx - c.ox;
+    if (xsend) {
+      const int sub = zoff / nz, xl = nbr[6 * sub], xr = nbr[6 * sub + 1];
+      const long long nloc = sz * nz, h = nx - ox;
       dr = (long long)(xr - sub) * nloc - h;
       dl = (long long)(xl - sub) * nloc + h;
 #pragma unroll
       for (int i = 0; i < V; ++i) {
         if (!xyin[i]) continue;
-        if (xr >= 0 && xs + i == nx - c.ox) sendm |= 1u << i;
-        if (xl >= 0 && xs + i == c.ox - 1) sendm |= 1u << (8 + i);
+        if (xr >= 0 && xs + i == nx - ox) sendm |= 1u << i;
+        if (xl >= 0 && xs + i == ox - 1) sendm |= 1u << (8 + i);
       }
     }
     int rb[Sh::RPT];
@@ -500,7 +500,7 @@ __global__ void __launch_bounds__(32 * GpShape<S>::WARPS, 1)
           const S xp = i == V - 1 ? wr : tc[i + 1];
           const S uc = WHICH == 0 ? ov.v[i] : tc[i], vc = WHICH == 0 ? tc[i] : ov.v[i];
           res[i] = gp_out_f32(ov.v[i], uc, vc, pv.v[i], tc[i], xm, xp, wym.v[i], wyp.v[i], tm[i],
-                              tp[i], c, WHICH);
+                              tp[i], pw, WHICH);
         }
       }
       const long long p0 = zoff * sz + xs + (long long)nx * y + sz * z;
@@ -586,7 +586,8 @@ cudaError_t launch_tma(int nsub, int nx, int ny, int nz, void *u, void *v, const
   const long long U = ncol * (nz - 2);
   const long long G = std::min<long long>((long long)per_sm * sms, std::max<long long>(1, U / 4));
   k_gp_tma<S, WHICH><<<(unsigned)G, 32 * Sh::WARPS, Sh::SMEM, s>>>(
-      mW, mO, mV, nx, ny, nz, ncx, ncx * ncy, (int)ncol, (S *)o, c, dev_err);
+      mW, mO, mV, nx, ny, nz, ncx, ncx * ncy, (int)ncol, (S *)o, make_gp_w(c, WHICH), c.nbr, c.ox,
+      c.xsend, dev_err);
   return cudaGetLastError();
 }
 
@@ -599,7 +600,7 @@ cudaError_t launch_w(int nsub, int nx, int ny, int nz, void *u, void *v, const v
   if (gz > 65535 || nx < 3) return cudaErrorInvalidValue;
   const dim3 grid((nx - 2 + kGpX - 1) / kGpX, (ny_in + kGpY - 1) / kGpY, (unsigned)gz);
   k_gp_half<S, WHICH><<<grid, dim3(kGpX, kGpY), 0, s>>>(nx, ny, nz, zchunks, (S *)u, (S *)v,
-                                                       (const S *)V, c);
+                                                       (const S *)V, make_gp_w(c, WHICH));
   return cudaGetLastError();
 }
 

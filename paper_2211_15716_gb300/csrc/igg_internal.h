@@ -38,7 +38,17 @@ constexpr int kTileY = 8;
 // all formed on the host in FP64.
 struct Coef {
   double wx, wy, wz, wc;
+  // the same (x, y, z, centre) as float pairs wh + wl and scaled copies of
+  // them, ah, al = 2^23 wh, 2^23 wl, for the kernels' FP32 and float-pair sums.
+  // Formed on the host: kernel arguments sit in the constant bank, whereas
+  // conversions at the head of a kernel were repeated inside its loop where
+  // registers ran short, on the FP64 pipe (two instructions per SM and clock):
+  // 2x2x2 x 512x256x256, ten steps, FP64 11.23 to 11.03 ms, BF16 3.36 to 3.30;
+  // 2x2x2 x 255x127x129 FP64, ten steps, 2.89 to 2.57 ms; the misfit gradient
+  // at 256^3 FP64, 48 steps, 22.9 to 22.5 ms.
+  float wh[4], wl[4], ah[4], al[4];
   int f64_emu;  // FP64 fields: 1 = emulated FP64 cell, 0 = FP64 cell
+  int pair;     // wx, wy, wz in the range of the adjoint's float-pair path (adj_cell.cuh)
   // TMA full steps followed by a halo update: the row end cells x = 0 and
   // x = n_x - 1 of every computed row are stored as well, with their values
   // in T (boundary cells keep them; halo cells are overwritten by the halo

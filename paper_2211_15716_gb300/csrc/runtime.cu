@@ -53,6 +53,15 @@ Coef make_coef(double lam, double dt, double dx, double dy, double dz) {
   c.wy = k / (dy * dy);
   c.wz = k / (dz * dz);
   c.wc = -2.0 * (c.wx + c.wy + c.wz);
+  const double w[4] = {c.wx, c.wy, c.wz, c.wc};
+  for (int i = 0; i < 4; ++i) {
+    c.wh[i] = (float)w[i];
+    c.wl[i] = (float)(w[i] - (double)c.wh[i]);
+    c.ah[i] = 8388608.0f * c.wh[i];
+    c.al[i] = 8388608.0f * c.wl[i];
+  }
+  c.pair = 1;
+  for (int i = 0; i < 3; ++i) c.pair = c.pair && w[i] >= 0x1p-18 && w[i] <= 0x1p18;
   c.f64_emu = 0;
   c.ends = 0;
   c.npts = 0;
