@@ -368,21 +368,12 @@ __device__ __forceinline__ bool emu2_centre_ok(unsigned hc) {
   return (hc & 0x7FF00000u) - (180u << 20) < (1829u << 20);
 }
 
-// Integer part of the fast path for one point: the group sums of the bit-
-// pattern second differences, split into the bits gh of the FP32 number
-// 1.5 2^23 + Gh and the bits gm of the FP32 number 1.5 2^23 + Gl. True when
-// the seven values share sign and exponent and every Gh lies in
-// [-2^22, 2^22), i.e. gh in [0x4B000000, 0x4B800000) (the centre's own test
-// is emu2_centre_ok). nb: x-, x+, y-, y+, z-, z+.
+// The group sums G_g + B (mod 2^64) of the second differences of 64-bit
+// integers: centre c, neighbours nb (x-, x+, y-, y+, z-, z+).
 template <int NG>
-__device__ __forceinline__ bool emu2_int(unsigned long long bc, const unsigned long long *nb,
-                                         unsigned *gh, unsigned *gm) {
-  const unsigned hc = (unsigned)(bc >> 32);
-  unsigned o = 0u;
-#pragma unroll
-  for (int i = 0; i < 6; ++i) o |= (unsigned)(nb[i] >> 32) ^ hc;
-  const unsigned long long c2 = bc << 1, B = 1ull << 22;
-  unsigned long long G[NG];  // G_g + 2^22 (mod 2^64)
+__device__ __forceinline__ void emu2_groups(unsigned long long c, const unsigned long long *nb,
+                                            unsigned long long B, unsigned long long *G) {
+  const unsigned long long c2 = c << 1;
   if constexpr (NG == 1) {
     G[0] = (nb[0] + nb[1] - c2) + (nb[2] + nb[3] - c2) + (nb[4] + nb[5] - c2) + B;
   } else if constexpr (NG == 2) {
@@ -392,7 +383,23 @@ __device__ __forceinline__ bool emu2_int(unsigned long long bc, const unsigned l
 #pragma unroll
     for (int d = 0; d < 3; ++d) G[d] = nb[2 * d] + nb[2 * d + 1] - c2 + B;
   }
-  unsigned r = 0u;
+}
+
+// Integer part of the fast path for one point: the group sums of the bit-
+// pattern second differences, split into the bits gh of the FP32 number
+// 1.5 2^23 + Gh and the bits gm of the FP32 number 1.5 2^23 + Gl. The tests'
+// terms are gathered in o and r: the neighbours share sign and exponent with
+// hc (a high word) when o < 2^20, and every Gh lies in [-2^22, 2^22), i.e. gh
+// in [0x4B000000, 0x4B800000), when r < 2^23 (the centre's own test is
+// emu2_centre_ok). nb: x-, x+, y-, y+, z-, z+.
+template <int NG>
+__device__ __forceinline__ void emu2_int(unsigned long long bc, const unsigned long long *nb,
+                                         unsigned hc, unsigned *gh, unsigned *gm, unsigned &o,
+                                         unsigned &r) {
+#pragma unroll
+  for (int i = 0; i < 6; ++i) o |= (unsigned)(nb[i] >> 32) ^ hc;
+  unsigned long long G[NG];  // G_g + 2^22 (mod 2^64)
+  emu2_groups<NG>(bc, nb, 1ull << 22, G);
 #pragma unroll
   for (int g = 0; g < NG; ++g) {
     const unsigned lo = (unsigned)G[g];
@@ -400,7 +407,6 @@ __device__ __forceinline__ bool emu2_int(unsigned long long bc, const unsigned l
     gm[g] = (lo & 0x7FFFFFu) | 0x4B000000u;
     r |= gh[g] ^ 0x4B000000u;
   }
-  return o < (1u << 20) && r < (1u << 23);
 }
 
 // S + C = sum_g w_g G_g from the FP32 halves (per lane: one point or two);
@@ -436,8 +442,8 @@ __device__ __forceinline__ void emu2_sum(const V *gh, const V *gl, const W<doubl
   }
 }
 
-// Ci truncated to an FP32 number (meaningful when emu2_apply's Ci condition
-// holds: Ci positive with its exponent field in [897, 1150]).
+// Ci truncated to an FP32 number (meaningful where the fast path's condition on
+// Ci holds: Ci positive with its exponent field in [897, 1150]).
 __device__ __forceinline__ float emu2_cif(double ci) {
   return __uint_as_float(__funnelshift_l((unsigned)__double2loint(ci),
                                          (unsigned)__double2hiint(ci) - (896u << 20), 3));
@@ -446,10 +452,9 @@ __device__ __forceinline__ float emu2_cif(double ci) {
 // T2 of a fast-path point from S and Kr = fma(Ci_f, C, 1.5 2^23) (one
 // rounding: the nearest integer to Ci_f C is bits(Kr) - 0x4B400000 when
 // |Ci_f C| < 2^22);
-// hc: the high word that gives the point's sign and exponent (see above);
-// ok is cleared where the remaining conditions fail.
+// hc: the high word that gives the point's sign and exponent (see above).
 __device__ __forceinline__ double emu2_apply(unsigned long long bc, unsigned hc, double ci,
-                                             float S, float Kr, bool &ok) {
+                                             float S, float Kr) {
   const unsigned sb = __float_as_uint(S);
   const unsigned eoff = (hc & 0x7FF00000u) - (179u << 20);
   const double sd = __hiloint2double((int)(((sb << 1) >> 4) + eoff), (int)(sb << 29));
@@ -458,9 +463,15 @@ __device__ __forceinline__ double emu2_apply(unsigned long long bc, unsigned hc,
   const double t2 = __fma_rn(sci, sd, __longlong_as_double((long long)bc));
   const unsigned long long r =
       dbits(t2) + (unsigned long long)__float_as_uint(Kr) - 0x4B400000ull;
-  ok = ok && cih - (897u << 20) < (254u << 20) && fabsf(Kr - kMagic) < 4194304.0f &&
-       (((unsigned)(r >> 32) ^ (unsigned)(bc >> 32)) & 0xFFF00000u) == 0u;
   return __longlong_as_double((long long)r);
+}
+
+// The fast path's conditions besides the centre's: the terms o (the result's
+// high word included) and r of emu2_int, Ci positive in the FP32 range, and the
+// correction's range (K = Kr - 1.5 2^23).
+__device__ __forceinline__ bool emu2_ok(unsigned o, unsigned r, double ci, float K) {
+  return o < (1u << 20) && r < (1u << 23) && dhi(ci) - (897u << 20) < (254u << 20) &&
+         fabsf(K) < 4194304.0f;
 }
 
 // The fast path for one point; ok tells whether it applies.
@@ -468,8 +479,9 @@ template <int NG>
 __device__ __forceinline__ double cell_emu_fast(double tc, const unsigned long long *nb,
                                                 double ci, const W<double> &w, bool &ok) {
   const unsigned long long bc = dbits(tc);
-  unsigned gh[NG], gm[NG];
-  ok = emu2_int<NG>(bc, nb, gh, gm) && emu2_centre_ok((unsigned)(bc >> 32));
+  const unsigned hc = (unsigned)(bc >> 32);
+  unsigned gh[NG], gm[NG], o = 0u, r = 0u;
+  emu2_int<NG>(bc, nb, hc, gh, gm, o, r);
   float fh[NG], fl[NG];
 #pragma unroll
   for (int g = 0; g < NG; ++g) {
@@ -479,7 +491,10 @@ __device__ __forceinline__ double cell_emu_fast(double tc, const unsigned long l
   float S, C;
   emu2_sum<NG>(fh, fl, w, S, C);
   const float Kr = __fmaf_rn(emu2_cif(ci), C, kMagic);
-  return emu2_apply(bc, (unsigned)(bc >> 32), ci, S, Kr, ok);
+  const double t2 = emu2_apply(bc, hc, ci, S, Kr);
+  o |= dhi(t2) ^ hc;
+  ok = emu2_centre_ok(hc) && emu2_ok(o, r, ci, vadd(Kr, -kMagic));
+  return t2;
 }
 
 __device__ __forceinline__ double cell_emu_fast(double tc, const unsigned long long *nb,
@@ -530,19 +545,20 @@ __device__ __forceinline__ bool emu3_int(unsigned long long bc, const unsigned l
 #pragma unroll
   for (int i = 0; i < 6; ++i) e = max(e, (unsigned)(nb[i] >> 52) & 0x7FFu);
   er = max(e, 1u);
-  long long I[6];
+  const unsigned long long B = 1ull << 22;
+  unsigned long long G[NG];  // G_g + 2^22
+  unsigned o = 0u;
 #pragma unroll
-  for (int i = 0; i < 6; ++i) I[i] = emu3_aligned(nb[i], bc, er);
-  const long long c2 = 2 * emu3_aligned(bc, bc, er), B = 1ll << 22;
-  long long G[NG];  // G_g + 2^22
-  if constexpr (NG == 1) {
-    G[0] = (I[0] + I[1] - c2) + (I[2] + I[3] - c2) + (I[4] + I[5] - c2) + B;
-  } else if constexpr (NG == 2) {
-    G[0] = I[0] + I[1] - c2 + B;
-    G[1] = (I[2] + I[3] - c2) + (I[4] + I[5] - c2) + B;
+  for (int i = 0; i < 6; ++i) o |= (unsigned)(nb[i] >> 32) ^ (unsigned)(bc >> 32);
+  if (o < (1u << 20)) {
+    // all seven share sign and exponent (their differences are too large for the
+    // fast path): the bit patterns differ as the aligned integers do
+    emu2_groups<NG>(bc, nb, B, G);
   } else {
+    unsigned long long I[6];
 #pragma unroll
-    for (int d = 0; d < 3; ++d) G[d] = I[2 * d] + I[2 * d + 1] - c2 + B;
+    for (int i = 0; i < 6; ++i) I[i] = (unsigned long long)emu3_aligned(nb[i], bc, er);
+    emu2_groups<NG>((unsigned long long)emu3_aligned(bc, bc, er), I, B, G);
   }
   unsigned r = 0u;
 #pragma unroll
@@ -594,20 +610,6 @@ __device__ __forceinline__ double cell_emu(double tc, const double *tn, double c
   double r = cell_emu_fast(tc, nb, ci, w, ok);
   if (ok) return r;
   r = cell_emu_aligned(tc, nb, ci, w, ok);
-  if (ok) return r;
-  return cell_f64(tc, tn[0], tn[1], tn[2], tn[3], tn[4], tn[5], ci, w);
-}
-
-// cell_emu of a point whose fast path is known not to apply (the points a
-// kernel left to its fix-up): the aligned path, else cell_f64.
-__device__ __forceinline__ double cell_emu_not_fast(double tc, const double *tn, double ci,
-                                                    const W<double> &w) {
-  if (!w.emu) return cell_f64(tc, tn[0], tn[1], tn[2], tn[3], tn[4], tn[5], ci, w);
-  unsigned long long nb[6];
-#pragma unroll
-  for (int i = 0; i < 6; ++i) nb[i] = dbits(tn[i]);
-  bool ok;
-  const double r = cell_emu_aligned(tc, nb, ci, w, ok);
   if (ok) return r;
   return cell_f64(tc, tn[0], tn[1], tn[2], tn[3], tn[4], tn[5], ci, w);
 }

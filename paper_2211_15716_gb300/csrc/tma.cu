@@ -115,6 +115,9 @@ __host__ __device__ constexpr bool is_emu(int mode) {
   return mode >= MODE_EMU && mode <= MODE_EMU_LAST;
 }
 constexpr int emu_mode(int ng) { return MODE_EMU + 3 - ng; }
+__host__ __device__ constexpr int emu_groups(int mode) {
+  return is_emu(mode) ? MODE_EMU + 3 - mode : 3;
+}
 
 // V points of one row: centre vector c, x neighbours from c and the points
 // beyond it (left, right), y and z neighbour vectors. ok gets bit i for each
@@ -166,10 +169,10 @@ __device__ __forceinline__ void compute_vec_emu(
   unsigned gh0[NG], gh1[NG], gm0[NG], gm1[NG];
   // sign and exponent from the pair's first point (shared by every point of
   // the pair whose stencil passes)
-  const unsigned hc = (unsigned)(b0 >> 32);
-  const bool okc = emu2_centre_ok(hc);
-  bool ok0 = emu2_int<NG>(b0, nb0, gh0, gm0) && okc;
-  bool ok1 = emu2_int<NG>(b1, nb1, gh1, gm1) && okc;
+  const unsigned hc = (unsigned)(b0 >> 32), hc1 = (unsigned)(b1 >> 32);
+  unsigned o0 = 0u, r0 = 0u, o1 = 0u, r1 = 0u;
+  emu2_int<NG>(b0, nb0, hc, gh0, gm0, o0, r0);
+  emu2_int<NG>(b1, nb1, hc1, gh1, gm1, o1, r1);
   // the FP32 sums of both points as float2 (one instruction per pair)
   float2 fh[NG], fl[NG];
 #pragma unroll
@@ -183,9 +186,16 @@ __device__ __forceinline__ void compute_vec_emu(
   emu2_sum<NG>(fh, fl, w, S, C);
   const float2 Kr = vfma(make_float2(emu2_cif(ci.v[0]), emu2_cif(ci.v[1])), C,
                          vset(kMagic, float2()));
-  out.v[0] = emu2_apply(b0, hc, ci.v[0], S.x, Kr.x, ok0);
-  out.v[1] = emu2_apply(b1, hc, ci.v[1], S.y, Kr.y, ok1);
-  ok = (ok0 ? 1u : 0u) | (ok1 ? 2u : 0u);
+  out.v[0] = emu2_apply(b0, hc, ci.v[0], S.x, Kr.x);
+  out.v[1] = emu2_apply(b1, hc, ci.v[1], S.y, Kr.y);
+  // the results keep the exponent too: one comparison with the neighbours'
+  o0 |= dhi(out.v[0]) ^ hc;
+  o1 |= dhi(out.v[1]) ^ hc1;
+  const float2 K = vadd(Kr, vset(-kMagic, float2()));
+  const bool okc = emu2_centre_ok(hc);
+  const bool p0 = okc && emu2_ok(o0, r0, ci.v[0], K.x);
+  const bool p1 = okc && emu2_ok(o1, r1, ci.v[1], K.y);
+  ok = (p0 ? 1u : 0u) | (p1 ? 2u : 0u);
 }
 template <>
 __device__ __forceinline__ void compute_vec<double, MODE_EMU>(
@@ -347,10 +357,9 @@ __global__ void __launch_bounds__(32 * 9, IGG_TMA_MIN_BLOCKS)
       }
       __syncwarp();
     };
-    // FP64: two march steps per iteration (the z-plane registers alternate
-    // instead of being copied; measured faster by a few percent)
-    constexpr int kUnroll = sizeof(S) == 8 ? 2 : 1;
-#pragma unroll kUnroll
+    // (not unrolled: two copies of the body spilled at the register budget; ten
+    // steps of 2x2x2 x 512x256x256 FP64 11.03, with one 10.36 ms)
+#pragma unroll 1
     for (int m = t.m0; ok && m < t.m1; ++m) {
       const int k = m - t.m0 + 1;
       const int s = k % NS, s1 = (k + 1) % NS;
@@ -466,16 +475,27 @@ __global__ void __launch_bounds__(32 * 9, IGG_TMA_MIN_BLOCKS)
 // as every kernel: the aligned path for stencils across powers of two or
 // zero, else the FP64 cell). The kernel listed every 32-point row segment
 // with such points (its first point and a bit mask). Each warp takes
-// kFixBatch entries at a time (one per lane of lanes 0..kFixBatch-1) and
-// deals their listed points out to its lanes, 32 at a time, in the order of
-// the entries and their bits, so that lanes are not left idle by sparse
-// masks. Each block adds its segments and points to the list's totals; the
-// last block to finish resets the list.
+// kFixBatch entries at a time (one per lane of lanes 0..kFixBatch-1). Entries
+// with kFixDense points or more go a lane per point of the segment (contiguous
+// loads); the others' listed points are dealt out to the lanes, 32 at a time,
+// in the order of the entries and their bits, so that lanes are not left idle
+// by sparse masks. The points that need the FP64 cell wait in a queue of the
+// warp until 32 of them are there: its eight FP64 instructions hold the SM's
+// FP64 pipe for 128 cycles however few lanes need them, and where a tenth of
+// the points did, nearly every round had some.
+// On a sign-changing field (2x2x2 x 256x128x128, modes up to 8: 80 % of the
+// points listed, a tenth of them FP64), twenty steps: 14.3 to 12.3 ms with the
+// queue, the dense entries and the aligned path's same-exponent form.
+// Each block adds its segments and points to the list's totals; the last
+// block to finish resets the list.
 constexpr unsigned kFixBatch = 4;
+constexpr int kFixDense = 16;
+template <int NG>
 __global__ void __launch_bounds__(256)
     k_fixup_f64(void *__restrict__ fix, size_t cap, double *__restrict__ T2,
                 const double *__restrict__ T, const double *__restrict__ Ci, int nx, int ny,
                 Coef c0) {
+  __shared__ long long queue[8][64];
   const FixList fl = fix_list(fix, cap);
   const unsigned count = (unsigned)min((size_t)*(volatile unsigned *)fl.count, cap);
   const W<double> w = make_w(c0, 0.0);
@@ -483,11 +503,73 @@ __global__ void __launch_bounds__(256)
   const int lane = threadIdx.x & 31;
   const unsigned warps = gridDim.x * (blockDim.x >> 5);
   const unsigned gw = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  long long *que = queue[threadIdx.x >> 5];
+  unsigned nque = 0u;  // warp-uniform
   unsigned segs = 0u, pts = 0u;
+  auto stencil = [&](long long p, double *tn) {
+    tn[0] = __ldg(T + p - 1);
+    tn[1] = __ldg(T + p + 1);
+    tn[2] = __ldg(T + p - sy);
+    tn[3] = __ldg(T + p + sy);
+    tn[4] = __ldg(T + p - sz);
+    tn[5] = __ldg(T + p + sz);
+  };
+  // the FP64 cell for the first n queued points
+  auto run_queue = [&](unsigned n) {
+    __syncwarp();
+    if ((unsigned)lane < n) {
+      const long long p = que[lane];
+      double tn[6];
+      stencil(p, tn);
+      T2[p] = cell_f64(__ldg(T + p), tn[0], tn[1], tn[2], tn[3], tn[4], tn[5], __ldg(Ci + p), w);
+    }
+    __syncwarp();
+  };
   for (unsigned b = gw * kFixBatch; b < count; b += warps * kFixBatch) {
     FixEntry en = {};
     if (lane < (int)kFixBatch && b + lane < count) en = fl.e[b + lane];
-    // inclusive prefix of the entries' point counts over lanes 0..kFixBatch-1
+    segs += __popc(__ballot_sync(0xffffffffu, en.bits != 0u));
+    pts += __reduce_add_sync(0xffffffffu, (unsigned)__popc(en.bits));
+    // one point per lane, the point at p where `on`
+    auto round = [&](bool on, long long p) {
+      bool f64 = false;
+      if (on && in_bounds(p - sz, c0.npts) && in_bounds(p + sz, c0.npts)) {
+        double tn[6];
+        stencil(p, tn);
+        const double tc = __ldg(T + p), ci = __ldg(Ci + p);
+        unsigned long long nb[6];
+#pragma unroll
+        for (int i = 0; i < 6; ++i) nb[i] = dbits(tn[i]);
+        bool ok;
+        const double v = cell_emu_aligned<NG>(tc, nb, ci, w, ok);
+        if (ok) T2[p] = v;
+        f64 = !ok;
+      }
+      const unsigned m = __ballot_sync(0xffffffffu, f64);
+      if (m) {
+        if (f64) que[nque + __popc(m & ((1u << lane) - 1u))] = p;
+        nque += __popc(m);
+        if (nque >= 32u) {
+          run_queue(32u);
+          nque -= 32u;
+          if ((unsigned)lane < nque) que[lane] = que[32 + lane];
+          __syncwarp();  // the moved entries before the next ones
+        }
+      }
+    };
+    // dense entries (kFixDense points and more): a lane per point of the segment,
+    // its loads and stores contiguous, without dealing
+    unsigned dense = __ballot_sync(0xffffffffu, __popc(en.bits) >= kFixDense);
+    while (dense) {
+      const int q = __ffs(dense) - 1;
+      dense &= dense - 1u;
+      const unsigned bits = __shfl_sync(0xffffffffu, en.bits, q);
+      const long long p0 = __shfl_sync(0xffffffffu, en.p, q);
+      round((bits >> lane & 1u) != 0u, p0 + lane);
+    }
+    if (__popc(en.bits) >= kFixDense) en.bits = 0u;
+    // the others: inclusive prefix of the entries' point counts over lanes
+    // 0..kFixBatch-1
     unsigned pre = __popc(en.bits);
 #pragma unroll
     for (unsigned d = 1; d < kFixBatch; d <<= 1) {
@@ -495,8 +577,7 @@ __global__ void __launch_bounds__(256)
       if ((unsigned)lane >= d) pre += v;
     }
     const unsigned total = __shfl_sync(0xffffffffu, pre, kFixBatch - 1);
-    segs += __popc(__ballot_sync(0xffffffffu, en.bits != 0u));
-    pts += total;
+    if (total == 0u) continue;
     unsigned pk[kFixBatch], bk[kFixBatch];
     long long qk[kFixBatch];
 #pragma unroll
@@ -506,8 +587,7 @@ __global__ void __launch_bounds__(256)
       qk[q] = __shfl_sync(0xffffffffu, en.p, q);
     }
     for (unsigned r = 0; r < total; r += 32u) {
-      const unsigned rank = r + lane;
-      if (rank >= total) break;
+      const unsigned rank = min(r + lane, total - 1u);
       // the entry holding the point of this rank and the point's bit
       unsigned q = 0u;
 #pragma unroll
@@ -521,15 +601,10 @@ __global__ void __launch_bounds__(256)
           excl = pk[k - 1];
           p0 = qk[k];
         }
-      const long long p = p0 + __fns(bits, 0u, (int)(rank - excl + 1u));
-      if (in_bounds(p - sz, c0.npts) && in_bounds(p + sz, c0.npts)) {
-        const double tc = __ldg(T + p);
-        const double tn[6] = {__ldg(T + p - 1),  __ldg(T + p + 1),  __ldg(T + p - sy),
-                              __ldg(T + p + sy), __ldg(T + p - sz), __ldg(T + p + sz)};
-        T2[p] = cell_emu_not_fast(tc, tn, __ldg(Ci + p), w);
-      }
+      round(r + lane < total, p0 + __fns(bits, 0u, (int)(rank - excl + 1u)));
     }
   }
+  run_queue(nque);
   __shared__ unsigned bsum[2];
   if (threadIdx.x == 0) bsum[0] = bsum[1] = 0u;
   __syncthreads();
@@ -580,8 +655,8 @@ cudaError_t launch_t(const TmaTile *tiles, int ntiles, void *T2, const void *T, 
                                                           dev_err, fix.p, fix.cap);
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess && is_emu(MODE)) {
-    k_fixup_f64<<<kFixupBlocks, 256, 0, s>>>(fix.p, fix.cap, (double *)T2, (const double *)T,
-                                            (const double *)Ci, nx, ny, cc);
+    k_fixup_f64<emu_groups(MODE)><<<kFixupBlocks, 256, 0, s>>>(
+        fix.p, fix.cap, (double *)T2, (const double *)T, (const double *)Ci, nx, ny, cc);
     e = cudaGetLastError();
   }
   return e;
