@@ -37,7 +37,7 @@ __device__ __forceinline__ double v64_at(const double *__restrict__ lam_in,
 // runs every plane (the warp votes inside need all lanes); stores are masked.
 template <class S>
 __global__ void __launch_bounds__(kAdjX *kAdjY)
-    k_adjoint(int nx, int ny, int nz, int zb, S *__restrict__ lam_out,
+    k_adjoint(int nx, int ny, int nz, int zb, int zchunks, S *__restrict__ lam_out,
               const S *__restrict__ lam_in, const S *__restrict__ Tn,
               const S *__restrict__ Ci, double *__restrict__ gCi, Coef c) {
   using Ops = AdjOps<S>;
@@ -47,7 +47,14 @@ __global__ void __launch_bounds__(kAdjX *kAdjY)
   const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * kAdjX + tx;
   const int x0 = blockIdx.x * kAdjX, y0 = blockIdx.y * kAdjY;
   const int x = x0 + tx, y = y0 + ty;
-  const int z0 = blockIdx.z * zb, z1 = min(z0 + zb, nz);
+  // blockIdx.z = subdomain * zchunks + z chunk
+  const long long base = (long long)(blockIdx.z / zchunks) * nx * ny * nz;
+  lam_out += base;
+  lam_in += base;
+  Tn += base;
+  Ci += base;
+  gCi += base;
+  const int z0 = (int)(blockIdx.z % zchunks) * zb, z1 = min(z0 + zb, nz);
   const typename Ops::WT aw = Ops::weights(c);
   const long long sy = nx, sz = (long long)nx * ny;
   // ring position of this thread (tid < kAdjRing): rows y0-1 and y0+kAdjY
@@ -141,24 +148,25 @@ __global__ void __launch_bounds__(256)
 
 }  // namespace
 
-cudaError_t launch_adjoint(igg_dtype dt, int nx, int ny, int nz, void *lam_out,
+cudaError_t launch_adjoint(igg_dtype dt, int nsub, int nx, int ny, int nz, void *lam_out,
                            const void *lam_in, const void *Tn, const void *Ci, double *gCi,
                            const Coef &c, bool tma, unsigned *dev_err, cudaStream_t s,
                            const void *ci_pairs) {
   if (tma && adjoint_tma_applies(dt, nx, lam_out, lam_in, Tn, Ci, gCi))
-    return launch_adjoint_tma(dt, nx, ny, nz, lam_out, lam_in, Tn, Ci, gCi, c, dev_err, s,
+    return launch_adjoint_tma(dt, nsub, nx, ny, nz, lam_out, lam_in, Tn, Ci, gCi, c, dev_err, s,
                               dt == IGG_F64 ? ci_pairs : nullptr);
-  const int zb = std::min(nz, 32);
-  const dim3 grid((nx + kAdjX - 1) / kAdjX, (ny + kAdjY - 1) / kAdjY, (nz + zb - 1) / zb);
+  const int zb = std::min(nz, 32), zc = (nz + zb - 1) / zb;
+  if ((long long)nsub * zc > 65535) return cudaErrorInvalidValue;
+  const dim3 grid((nx + kAdjX - 1) / kAdjX, (ny + kAdjY - 1) / kAdjY, (unsigned)(nsub * zc));
   const dim3 block(kAdjX, kAdjY);
   switch (dt) {
     case IGG_F64:
-      k_adjoint<double><<<grid, block, 0, s>>>(nx, ny, nz, zb, (double *)lam_out,
+      k_adjoint<double><<<grid, block, 0, s>>>(nx, ny, nz, zb, zc, (double *)lam_out,
                                                (const double *)lam_in, (const double *)Tn,
                                                (const double *)Ci, gCi, c);
       break;
     case IGG_F32:
-      k_adjoint<float><<<grid, block, 0, s>>>(nx, ny, nz, zb, (float *)lam_out,
+      k_adjoint<float><<<grid, block, 0, s>>>(nx, ny, nz, zb, zc, (float *)lam_out,
                                               (const float *)lam_in, (const float *)Tn,
                                               (const float *)Ci, gCi, c);
       break;

@@ -1,13 +1,16 @@
-// TMA-pipelined adjoint step over every point of one array (the transposed
+// TMA-pipelined adjoint step over every point of every subdomain (the transposed
 // stencil of Fig. 1's step! and the Ci-gradient increment; arithmetic in
 // adj_cell.cuh, the same bits as the tiled kernel of adjoint.cu).
 //
 // Tiles are W x H (x, y) columns (W = 32 lanes x one 16-byte vector: 64
 // FP64 or 128 FP32 points; H = 8 FP64 / 16 FP32 rows, one warp per row)
 // marching along z. A persistent grid (all CTAs resident) takes equal shares
-// of the work order (z chunk, column, plane), so every CTA handles the same
-// number of planes; a share splits into segments (runs of planes of one
-// column).
+// of the work order (z chunk, column of a subdomain, plane), so every CTA
+// handles the same number of planes; a share splits into segments (runs of
+// planes of one column). All subdomains go in one launch: with a launch each,
+// eight subdomains of 64^3 left most of the GPU idle eight times over
+// (FP32
+// misfit gradient of 32 steps there: 4.72 to 2.49 ms).
 //
 // Per plane p, cp.async.bulk.tensor (TMA) loads into a ring of NS shared-
 // memory stages the (W + 2V) x (H + 2) boxes of lam_in, Ci and T_n around the
@@ -80,7 +83,7 @@ template <class S, bool CIP>
 __global__ void __launch_bounds__(32 * AdjShape<S>::WARPS, AdjShape<S>::MINB)
     k_adjoint_tma(const __grid_constant__ CUtensorMap mL, const __grid_constant__ CUtensorMap mC,
                   const __grid_constant__ CUtensorMap mT, const __grid_constant__ CUtensorMap mG,
-                  int nx, int ny, int nz, int ncx, int ncol, S *__restrict__ lam_out,
+                  int nx, int ny, int nz, int ncx, int ncxy, int ncol, S *__restrict__ lam_out,
                   const S *__restrict__ lam_in, const S *__restrict__ Ci,
                   double *__restrict__ gCi, Coef c, unsigned *__restrict__ dev_err) {
   using Sh = AdjShape<S>;
@@ -99,6 +102,13 @@ __global__ void __launch_bounds__(32 * AdjShape<S>::WARPS, AdjShape<S>::MINB)
   const long long U = (long long)ncol * nz;
   const long long u0 = U * blockIdx.x / gridDim.x, u1 = U * (blockIdx.x + 1) / gridDim.x;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  // column col: tile origin and the first plane of its subdomain
+  auto origin = [&](int col, int &x0, int &r0, int &zoff) {
+    const int sub = col / ncxy, cc = col - sub * ncxy;
+    x0 = (cc % ncx) * W;
+    r0 = (cc / ncx) * H;
+    zoff = sub * nz;
+  };
 
   // the load cursor (used by thread 0 only): the loads of a segment are its
   // planes m0 - 1 .. m1
@@ -113,11 +123,14 @@ __global__ void __launch_bounds__(32 * AdjShape<S>::WARPS, AdjShape<S>::MINB)
         cK = cs.m1 - cs.m0 + 2;
       }
       const int s = issued % NS;
-      const int x0 = (cs.col % ncx) * W, r0 = (cs.col / ncx) * H;
+      int x0, r0, zoff;
+      origin(cs.col, x0, r0, zoff);
       const bool g = cj >= 1 && cj <= cK - 2;  // gCi of planes m0 .. m1-1
       const unsigned bar = full0 + 8 * s, dst = sbase + s * Sh::STAGE;
       mbar_expect_tx(bar, 3 * Sh::FB + (g ? Sh::GB : 0));
-      const int p = cs.m0 - 1 + cj;
+      // (beside a subdomain's own planes: a neighbour's plane or, outside the
+      // stack, zeros; only boundary points see them, which use neither)
+      const int p = zoff + cs.m0 - 1 + cj;
       tma_load_3d(dst, &mL, x0 - V, r0 - 1, p, bar);
       tma_load_3d(dst + Sh::FBA, &mC, x0 - V, r0 - 1, p, bar);
       tma_load_3d(dst + 2 * Sh::FBA, &mT, x0 - V, r0 - 1, p, bar);
@@ -158,7 +171,9 @@ __global__ void __launch_bounds__(32 * AdjShape<S>::WARPS, AdjShape<S>::MINB)
   LT qc[V], qp[V];
   VT vm[V], vc[V], vp[V];
   while (!stop && sh.next(sg)) {
-    const int x0 = (sg.col % ncx) * W, r0 = (sg.col / ncx) * H;
+    int x0, r0, zoff;
+    origin(sg.col, x0, r0, zoff);
+    const long long base = sz * zoff;  // first element of the subdomain
     const int xs = x0 + lane * V, y = r0 + r;
     const bool yin = y >= 1 && y <= ny - 2, yown = y < ny;
     bool xyin[V];
@@ -293,7 +308,7 @@ __global__ void __launch_bounds__(32 * AdjShape<S>::WARPS, AdjShape<S>::MINB)
               // Ci of an inner point: from the box, or (pairs in the box)
               // from memory
               auto ci_at = [&](const S *Cb, int bb, int xx, int yy, int zz) -> double {
-                if constexpr (CIP) return Ci[xx + (long long)nx * yy + sz * zz];
+                if constexpr (CIP) return Ci[base + xx + (long long)nx * yy + sz * zz];
                 else return Cb[bb];
               };
               auto v64 = [&](int bb, int xx, int yy) {
@@ -301,7 +316,7 @@ __global__ void __launch_bounds__(32 * AdjShape<S>::WARPS, AdjShape<S>::MINB)
                 return in ? adj_v64(L[bb], ci_at(C, bb, xx, yy, m), true) : 0.0;
               };
               const bool inm = in3(x, y, m - 1), inp = in3(x, y, m + 1);
-              const long long pm = x + (long long)nx * y + sz * (m - 1);
+              const long long pm = base + x + (long long)nx * y + sz * (m - 1);
               out[i] = adj_out_f64(lc[i], v64(b, x, y), v64(b - 1, x - 1, y), v64(b + 1, x + 1, y),
                                    v64(b - BW, x, y - 1), v64(b + BW, x, y + 1),
                                    adj_v64(inm ? lam_in[pm] : 0.0, inm ? Ci[pm] : 0.0, inm),
@@ -311,7 +326,7 @@ __global__ void __launch_bounds__(32 * AdjShape<S>::WARPS, AdjShape<S>::MINB)
           }
         }
       }
-      const long long p0 = xs + (long long)nx * y + sz * m;
+      const long long p0 = base + xs + (long long)nx * y + sz * m;
       if (yown) {
         if (xs + V <= nx) {
           Vec<S> o;
@@ -396,16 +411,17 @@ cudaError_t prepare_adj_t(int *ctas_per_sm) {
 }
 
 template <class S, bool CIP>
-cudaError_t launch_adj_t(int nx, int ny, int nz, void *lam_out, const void *lam_in, const void *Tn,
+cudaError_t launch_adj_t(int nsub, int nx, int ny, int nz, void *lam_out, const void *lam_in, const void *Tn,
                          const void *Ci, const void *ci_box, double *gCi, const Coef &c,
                          unsigned *dev_err, cudaStream_t s) {
   using Sh = AdjShape<S>;
   CUtensorMap mL, mC, mT, mG;
   // the Ci box: FP64 values, or their pairs (8 bytes each, the same box)
-  if (!encode<S>(&mL, lam_in, nx, ny, nz, Sh::BW, Sh::BH, 1) ||
-      !encode<S>(&mC, ci_box, nx, ny, nz, Sh::BW, Sh::BH, 1) ||
-      !encode<S>(&mT, Tn, nx, ny, nz, Sh::BW, Sh::BH, 1) ||
-      !encode<double>(&mG, gCi, nx, ny, nz, Sh::W, Sh::H, 1))
+  const long long nzt = (long long)nsub * nz;
+  if (!encode<S>(&mL, lam_in, nx, ny, nzt, Sh::BW, Sh::BH, 1) ||
+      !encode<S>(&mC, ci_box, nx, ny, nzt, Sh::BW, Sh::BH, 1) ||
+      !encode<S>(&mT, Tn, nx, ny, nzt, Sh::BW, Sh::BH, 1) ||
+      !encode<double>(&mG, gCi, nx, ny, nzt, Sh::W, Sh::H, 1))
     return cudaErrorInvalidValue;
   int per_sm = 0, dev = 0, sms = 0;
   cudaError_t e = prepare_adj_t<S, CIP>(&per_sm);
@@ -414,11 +430,13 @@ cudaError_t launch_adj_t(int nx, int ny, int nz, void *lam_out, const void *lam_
   if (e != cudaSuccess) return e;
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
   const int ncx = (nx + Sh::W - 1) / Sh::W, ncy = (ny + Sh::H - 1) / Sh::H;
-  const long long U = (long long)ncx * ncy * nz;
+  const long long ncol = (long long)nsub * ncx * ncy;
+  if (ncol > (1ll << 30) || nzt > (1ll << 30)) return cudaErrorInvalidValue;
+  const long long U = ncol * nz;
   // every CTA gets at least a few planes; at most the resident CTAs
   const long long G = std::min<long long>((long long)per_sm * sms, std::max<long long>(1, U / 4));
   k_adjoint_tma<S, CIP><<<(unsigned)G, 32 * Sh::WARPS, Sh::SMEM, s>>>(
-      mL, mC, mT, mG, nx, ny, nz, ncx, ncx * ncy, (S *)lam_out, (const S *)lam_in,
+      mL, mC, mT, mG, nx, ny, nz, ncx, ncx * ncy, (int)ncol, (S *)lam_out, (const S *)lam_in,
       (const S *)Ci, gCi, c, dev_err);
   return cudaGetLastError();
 }
@@ -446,19 +464,19 @@ bool adjoint_tma_applies(igg_dtype dt, int nx, const void *lam_out, const void *
   return true;
 }
 
-cudaError_t launch_adjoint_tma(igg_dtype dt, int nx, int ny, int nz, void *lam_out,
+cudaError_t launch_adjoint_tma(igg_dtype dt, int nsub, int nx, int ny, int nz, void *lam_out,
                                const void *lam_in, const void *Tn, const void *Ci, double *gCi,
                                const Coef &c, unsigned *dev_err, cudaStream_t s,
                                const void *ci_pairs) {
   switch (dt) {
     case IGG_F64:
       if (ci_pairs)
-        return launch_adj_t<double, true>(nx, ny, nz, lam_out, lam_in, Tn, Ci, ci_pairs, gCi, c,
+        return launch_adj_t<double, true>(nsub, nx, ny, nz, lam_out, lam_in, Tn, Ci, ci_pairs, gCi, c,
                                           dev_err, s);
-      return launch_adj_t<double, false>(nx, ny, nz, lam_out, lam_in, Tn, Ci, Ci, gCi, c,
+      return launch_adj_t<double, false>(nsub, nx, ny, nz, lam_out, lam_in, Tn, Ci, Ci, gCi, c,
                                          dev_err, s);
     case IGG_F32:
-      return launch_adj_t<float, false>(nx, ny, nz, lam_out, lam_in, Tn, Ci, Ci, gCi, c,
+      return launch_adj_t<float, false>(nsub, nx, ny, nz, lam_out, lam_in, Tn, Ci, Ci, gCi, c,
                                         dev_err, s);
     default:
       return cudaErrorInvalidValue;

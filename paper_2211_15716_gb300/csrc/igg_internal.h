@@ -297,11 +297,12 @@ cudaError_t launch_halo_adjoint(size_t elem_size, const PlaneCopy *copies, int n
                                 void *field, int na, int nb, long long sa, long long sb,
                                 cudaStream_t s);
 
-// Adjoint step over every point of one array, and out = a - b elementwise.
+// Adjoint step over every point of nsub arrays one after the other, and
+// out = a - b elementwise.
 // With `tma`, fields that allow it take the TMA-pipelined kernel; FP64 fields
 // with `ci_pairs` (Ci as pairs from launch_pair_ci, n elements of 8 bytes)
 // load those instead of splitting Ci (same results).
-cudaError_t launch_adjoint(igg_dtype dt, int nx, int ny, int nz, void *lam_out,
+cudaError_t launch_adjoint(igg_dtype dt, int nsub, int nx, int ny, int nz, void *lam_out,
                            const void *lam_in, const void *Tn, const void *Ci, double *gCi,
                            const Coef &c, bool tma, unsigned *dev_err, cudaStream_t s,
                            const void *ci_pairs = nullptr);
@@ -309,7 +310,7 @@ cudaError_t launch_adjoint(igg_dtype dt, int nx, int ny, int nz, void *lam_out,
 // 16-byte aligned fields (and a driver with tensor maps).
 bool adjoint_tma_applies(igg_dtype dt, int nx, const void *lam_out, const void *lam_in,
                          const void *Tn, const void *Ci, const double *gCi);
-cudaError_t launch_adjoint_tma(igg_dtype dt, int nx, int ny, int nz, void *lam_out,
+cudaError_t launch_adjoint_tma(igg_dtype dt, int nsub, int nx, int ny, int nz, void *lam_out,
                                const void *lam_in, const void *Tn, const void *Ci, double *gCi,
                                const Coef &c, unsigned *dev_err, cudaStream_t s,
                                const void *ci_pairs = nullptr);

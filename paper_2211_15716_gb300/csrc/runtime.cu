@@ -1465,19 +1465,21 @@ static int check_adjoint_grid(const igg_grid *g, igg_dtype dt) {
   return IGG_OK;
 }
 
-// The transposed step S^T on every subdomain (one launch each); the
-// subdomains' fields are consecutive blocks of nloc points.
+// The transposed step S^T on every subdomain (one launch; groups of
+// subdomains where the tiled kernel's grid would exceed its limit).
 static cudaError_t adjoint_subdomains(igg_grid *g, igg_dtype dt, void *lam_out,
                                       const void *lam_in, const void *Tn, const void *Ci,
                                       double *gCi, const Coef &c, cudaStream_t s,
                                       const void *ci_pairs) {
   const size_t bytes = (size_t)g->nloc * dtype_size(dt);
+  const int group = std::max(1, 65535 / ((g->n[2] + 31) / 32));
   cudaError_t e = cudaSuccess;
-  for (int k = 0; k < g->nsub && e == cudaSuccess; ++k) {
+  for (int k = 0; k < g->nsub && e == cudaSuccess; k += group) {
     const size_t o = (size_t)k * bytes;
-    e = launch_adjoint(dt, g->n[0], g->n[1], g->n[2], (char *)lam_out + o,
-                       (const char *)lam_in + o, (const char *)Tn + o, (const char *)Ci + o,
-                       gCi + (size_t)k * g->nloc, c, g->tma_enabled, g->dev_err, s,
+    e = launch_adjoint(dt, std::min(group, g->nsub - k), g->n[0], g->n[1], g->n[2],
+                       (char *)lam_out + o, (const char *)lam_in + o, (const char *)Tn + o,
+                       (const char *)Ci + o, gCi + (size_t)k * g->nloc, c, g->tma_enabled,
+                       g->dev_err, s,
                        ci_pairs ? (const char *)ci_pairs + (size_t)k * g->nloc * 8 : nullptr);
   }
   return e;
