@@ -71,7 +71,7 @@ __device__ __forceinline__ void ac_put(S *p, S v, const AcSend &a, long long np,
 
 template <class S>
 __global__ void __launch_bounds__(kAcX *kAcY)
-    k_acoustic_v(int nx, int ny, int nz, int zchunks, const S *__restrict__ P, S *__restrict__ Vx,
+    k_acoustic_v(int nx, int ny, int nz, int zchunks, const S *P, S *__restrict__ Vx,
                  S *__restrict__ Vy, S *__restrict__ Vz, AcCoef c) {
   using N = AcNum<S>;
   const int i = blockIdx.x * kAcX + threadIdx.x, j = blockIdx.y * kAcY + threadIdx.y;
@@ -100,6 +100,8 @@ __global__ void __launch_bounds__(kAcX *kAcY)
     keep = !((i == 0 && xl >= 0) || (i == nx - 1 && xr >= 0));
   }
   const bool sv = ev.sm != 0u;  // sends Vy and Vz (wall faces too)
+  pdl_trigger();
+  pdl_wait();
   S pzm = k0 > 0 ? Ps[sp * (k0 - 1)] : S(0);
   // plane k0
   S pc = Ps[sp * k0];
@@ -157,8 +159,7 @@ __global__ void __launch_bounds__(kAcX *kAcY)
 template <class S>
 __global__ void __launch_bounds__(kAcX *kAcY)
     k_acoustic_p(int nx, int ny, int nz, int zchunks, S *__restrict__ P,
-                 const S *__restrict__ Vx, const S *__restrict__ Vy, const S *__restrict__ Vz,
-                 AcCoef c) {
+                 const S *Vx, const S *Vy, const S *Vz, AcCoef c) {
   using N = AcNum<S>;
   const int i = blockIdx.x * kAcX + threadIdx.x, j = blockIdx.y * kAcY + threadIdx.y;
   if (i >= nx || j >= ny) return;
@@ -180,6 +181,8 @@ __global__ void __launch_bounds__(kAcX *kAcY)
     ep = ac_send(i, nx, c.ox, sub, xl, xr);
     keep = !((i == 0 && xl >= 0) || (i == nx - 1 && xr >= 0));
   }
+  pdl_trigger();
+  pdl_wait();
   S vzc = Vzs[sp * k0];
   // plane k0
   S pc = Ps[sp * k0], x0 = Vxs[sx * k0], x1 = Vxs[sx * k0 + 1], y0 = Vys[sy * k0],
@@ -221,13 +224,11 @@ cudaError_t launch_t(int nsub, int nx, int ny, int nz, void *P, void *Vx, void *
   if (gz > 65535) return cudaErrorInvalidValue;
   const dim3 grid((nx + kAcX - 1) / kAcX, (ny + kAcY - 1) / kAcY, (unsigned)gz);
   const dim3 block(kAcX, kAcY);
-  k_acoustic_v<S><<<grid, block, 0, s>>>(nx, ny, nz, zchunks, (const S *)P, (S *)Vx, (S *)Vy,
-                                          (S *)Vz, c);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = launch_pdl(true, k_acoustic_v<S>, grid, block, 0, s, nx, ny, nz, zchunks, (const S *)P,
+                             (S *)Vx, (S *)Vy, (S *)Vz, c);
   if (e != cudaSuccess) return e;
-  k_acoustic_p<S><<<grid, block, 0, s>>>(nx, ny, nz, zchunks, (S *)P, (const S *)Vx,
-                                          (const S *)Vy, (const S *)Vz, c);
-  return cudaGetLastError();
+  return launch_pdl(true, k_acoustic_p<S>, grid, block, 0, s, nx, ny, nz, zchunks, (S *)P, (const S *)Vx,
+                    (const S *)Vy, (const S *)Vz, c);
 }
 
 }  // namespace

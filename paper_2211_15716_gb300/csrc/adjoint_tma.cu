@@ -84,8 +84,7 @@ __global__ void __launch_bounds__(32 * AdjShape<S>::WARPS, AdjShape<S>::MINB)
     k_adjoint_tma(const __grid_constant__ CUtensorMap mL, const __grid_constant__ CUtensorMap mC,
                   const __grid_constant__ CUtensorMap mT, const __grid_constant__ CUtensorMap mG,
                   int nx, int ny, int nz, int ncx, int ncxy, int ncol, S *__restrict__ lam_out,
-                  const S *__restrict__ lam_in, const S *__restrict__ Ci,
-                  double *__restrict__ gCi, Coef c, unsigned *__restrict__ dev_err) {
+                  const S *lam_in, const S *Ci, double *__restrict__ gCi, Coef c, unsigned *__restrict__ dev_err) {
   using Sh = AdjShape<S>;
   using Ops = AdjOps<S>;
   using VT = typename Sh::VT;
@@ -144,6 +143,8 @@ __global__ void __launch_bounds__(32 * AdjShape<S>::WARPS, AdjShape<S>::MINB)
     for (int s = 0; s < NS; ++s) mbar_init(full0 + 8 * s, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    pdl_trigger();
+    pdl_wait();  // (and the CTA's other accesses follow its first load)
     issue_upto(NS - 2);
   }
   __syncthreads();
@@ -435,10 +436,9 @@ cudaError_t launch_adj_t(int nsub, int nx, int ny, int nz, void *lam_out, const 
   const long long U = ncol * nz;
   // every CTA gets at least a few planes; at most the resident CTAs
   const long long G = std::min<long long>((long long)per_sm * sms, std::max<long long>(1, U / 4));
-  k_adjoint_tma<S, CIP><<<(unsigned)G, 32 * Sh::WARPS, Sh::SMEM, s>>>(
-      mL, mC, mT, mG, nx, ny, nz, ncx, ncx * ncy, (int)ncol, (S *)lam_out, (const S *)lam_in,
-      (const S *)Ci, gCi, c, dev_err);
-  return cudaGetLastError();
+  return launch_pdl(pdl_on((long long)nsub * nx * ny * nz), k_adjoint_tma<S, CIP>, (unsigned)G, 32 * Sh::WARPS, Sh::SMEM, s, mL, mC, mT, mG,
+                    nx, ny, nz, ncx, ncx * ncy, (int)ncol, (S *)lam_out, (const S *)lam_in,
+                    (const S *)Ci, gCi, c, dev_err);
 }
 
 // Ci as pairs (pair_ci), once per checkpointed run

@@ -337,6 +337,8 @@ __global__ void __launch_bounds__(32 * GpShape<S>::WARPS, 1)
     for (int s = 0; s < NS; ++s) mbar_init(full0 + 8 * s, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    pdl_trigger();
+    pdl_wait();  // (and the CTA's other accesses follow its first load)
     issue_upto(NS - 2);
   }
   __syncthreads();
@@ -585,10 +587,9 @@ cudaError_t launch_tma(int nsub, int nx, int ny, int nz, void *u, void *v, const
   if (ncol > (1ll << 30)) return cudaErrorInvalidValue;
   const long long U = ncol * (nz - 2);
   const long long G = std::min<long long>((long long)per_sm * sms, std::max<long long>(1, U / 4));
-  k_gp_tma<S, WHICH><<<(unsigned)G, 32 * Sh::WARPS, Sh::SMEM, s>>>(
-      mW, mO, mV, nx, ny, nz, ncx, ncx * ncy, (int)ncol, (S *)o, make_gp_w(c, WHICH), c.nbr, c.ox,
-      c.xsend, dev_err);
-  return cudaGetLastError();
+  return launch_pdl(pdl_on((long long)nsub * nx * ny * nz), k_gp_tma<S, WHICH>, (unsigned)G, 32 * Sh::WARPS, Sh::SMEM, s, mW, mO, mV, nx,
+                    ny, nz, ncx, ncx * ncy, (int)ncol, (S *)o, make_gp_w(c, WHICH), c.nbr, c.ox,
+                    c.xsend, dev_err);
 }
 
 template <class S, int WHICH>

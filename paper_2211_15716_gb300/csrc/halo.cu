@@ -22,6 +22,8 @@ __global__ void __launch_bounds__(256)
   const int ci = blockIdx.x / nb, b = blockIdx.x % nb;
   const PlaneCopy c = copies[ci];
   const long long rb = (long long)b * sb;
+  pdl_trigger();
+  pdl_wait();
   if (VEC) {
     const uint4 *src = reinterpret_cast<const uint4 *>(f + c.src + rb);
     uint4 *dst = reinterpret_cast<uint4 *>(f + c.dst + rb);
@@ -36,11 +38,8 @@ template <class E>
 cudaError_t launch_e(const PlaneCopy *copies, int ncopies, void *field, int na, int nb,
                      long long sa, long long sb, bool vec, cudaStream_t s) {
   const unsigned blocks = (unsigned)((long long)ncopies * nb);
-  if (vec)
-    k_halo_planes<E, true><<<blocks, 256, 0, s>>>(copies, (E *)field, na, nb, sa, sb);
-  else
-    k_halo_planes<E, false><<<blocks, 256, 0, s>>>(copies, (E *)field, na, nb, sa, sb);
-  return cudaGetLastError();
+  return launch_pdl(blocks <= 16384u, vec ? k_halo_planes<E, true> : k_halo_planes<E, false>, blocks, 256, 0, s,
+                    copies, (E *)field, na, nb, sa, sb);
 }
 
 // Several fields' copies of one dimension in one launch: blockIdx.y picks the
@@ -48,6 +47,8 @@ cudaError_t launch_e(const PlaneCopy *copies, int ncopies, void *field, int na, 
 // row) of it; blocks beyond a job's copies x rows exit.
 template <class E>
 __global__ void __launch_bounds__(256) k_halo_jobs(const HaloJobs jobs) {
+  pdl_trigger();
+  pdl_wait();
   const HaloJob &j = jobs.j[blockIdx.y];
   const long long blk = blockIdx.x;
   if (blk >= (long long)j.ncopies * j.nb) return;
@@ -101,6 +102,8 @@ __global__ void __launch_bounds__(256) k_halo_gather(E *__restrict__ f, const Ha
   const int s0 = (int)(blockIdx.x / rows);
   int row = (int)(blockIdx.x % rows);
   const long long sy = nx, sz = (long long)nx * ny;
+  pdl_trigger();
+  pdl_wait();
   if (row < 2 * ny + 2 * (nz - 2)) {
     int y, z;
     if (row < 2 * ny) {
@@ -170,6 +173,8 @@ __global__ void __launch_bounds__(256)
   const int ci = blockIdx.x / nb, b = blockIdx.x % nb;
   const PlaneCopy c = copies[ci];
   const long long rb = (long long)b * sb;
+  pdl_trigger();
+  pdl_wait();
   for (int a = threadIdx.x; a < na; a += blockDim.x) {
     const long long i = c.dst + rb + a * sa, j = c.src + rb + a * sa;
     atomicAdd(f + j, f[i]);
@@ -197,12 +202,11 @@ cudaError_t launch_halo_jobs(size_t elem_size, HaloJobs jobs, int njobs, cudaStr
   if (blocks >= (1ll << 31)) return cudaErrorInvalidValue;
   const dim3 grid((unsigned)blocks, (unsigned)njobs);
   switch (elem_size) {
-    case 8: k_halo_jobs<unsigned long long><<<grid, 256, 0, s>>>(jobs); break;
-    case 4: k_halo_jobs<unsigned int><<<grid, 256, 0, s>>>(jobs); break;
-    case 2: k_halo_jobs<unsigned short><<<grid, 256, 0, s>>>(jobs); break;
+    case 8: return launch_pdl(true, k_halo_jobs<unsigned long long>, grid, 256, 0, s, jobs);
+    case 4: return launch_pdl(true, k_halo_jobs<unsigned int>, grid, 256, 0, s, jobs);
+    case 2: return launch_pdl(true, k_halo_jobs<unsigned short>, grid, 256, 0, s, jobs);
     default: return cudaErrorInvalidValue;
   }
-  return cudaGetLastError();
 }
 
 cudaError_t launch_halo(size_t elem_size, const PlaneCopy *copies, int ncopies,
@@ -229,12 +233,12 @@ cudaError_t launch_halo_adjoint(size_t elem_size, const PlaneCopy *copies, int n
   if ((long long)ncopies * nb >= (1ll << 31)) return cudaErrorInvalidValue;
   const unsigned blocks = (unsigned)((long long)ncopies * nb);
   if (elem_size == 8)
-    k_halo_planes_adj<double><<<blocks, 256, 0, s>>>(copies, (double *)field, na, nb, sa, sb);
-  else if (elem_size == 4)
-    k_halo_planes_adj<float><<<blocks, 256, 0, s>>>(copies, (float *)field, na, nb, sa, sb);
-  else
-    return cudaErrorInvalidValue;
-  return cudaGetLastError();
+    return launch_pdl(blocks <= 16384u, k_halo_planes_adj<double>, blocks, 256, 0, s, copies, (double *)field, na, nb,
+                      sa, sb);
+  if (elem_size == 4)
+    return launch_pdl(blocks <= 16384u, k_halo_planes_adj<float>, blocks, 256, 0, s, copies, (float *)field, na, nb,
+                      sa, sb);
+  return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_halo_gather(size_t elem_size, void *field, const HaloGather &h,
@@ -248,21 +252,18 @@ cudaError_t launch_halo_gather(size_t elem_size, void *field, const HaloGather &
   const unsigned b = (unsigned)blocks;
   switch (elem_size) {
     case 8:
-      if (vec) k_halo_gather<unsigned long long, true><<<b, 256, 0, s>>>((unsigned long long *)field, h);
-      else k_halo_gather<unsigned long long, false><<<b, 256, 0, s>>>((unsigned long long *)field, h);
-      break;
+      return launch_pdl(pdl_on(h.nloc * h.nsub), vec ? k_halo_gather<unsigned long long, true>
+                            : k_halo_gather<unsigned long long, false>,
+                        b, 256, 0, s, (unsigned long long *)field, h);
     case 4:
-      if (vec) k_halo_gather<unsigned, true><<<b, 256, 0, s>>>((unsigned *)field, h);
-      else k_halo_gather<unsigned, false><<<b, 256, 0, s>>>((unsigned *)field, h);
-      break;
+      return launch_pdl(pdl_on(h.nloc * h.nsub), vec ? k_halo_gather<unsigned, true> : k_halo_gather<unsigned, false>, b, 256,
+                        0, s, (unsigned *)field, h);
     case 2:
-      if (vec) k_halo_gather<unsigned short, true><<<b, 256, 0, s>>>((unsigned short *)field, h);
-      else k_halo_gather<unsigned short, false><<<b, 256, 0, s>>>((unsigned short *)field, h);
-      break;
-    default:
-      return cudaErrorInvalidValue;
+      return launch_pdl(pdl_on(h.nloc * h.nsub), vec ? k_halo_gather<unsigned short, true>
+                            : k_halo_gather<unsigned short, false>,
+                        b, 256, 0, s, (unsigned short *)field, h);
   }
-  return cudaGetLastError();
+  return cudaErrorInvalidValue;
 }
 
 cudaError_t halo_bounds_flag(unsigned *out, bool clear) { return read_bounds_flag(out, clear); }

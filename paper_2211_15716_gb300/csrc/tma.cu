@@ -271,6 +271,10 @@ __global__ void __launch_bounds__(32 * 9, IGG_TMA_MIN_BLOCKS)
   if (warp == Sh::CONSUMERS) {
     // ---------------- producer ----------------
     if (lane == 0) {
+      // the earlier launches complete before the first load, and with it before
+      // the consumers' first store
+      pdl_trigger();
+      pdl_wait();
       int k = 0;
       for (; k < K; ++k) {
         const int s = k % NS;
@@ -492,10 +496,11 @@ constexpr unsigned kFixBatch = 4;
 constexpr int kFixDense = 16;
 template <int NG>
 __global__ void __launch_bounds__(256)
-    k_fixup_f64(void *__restrict__ fix, size_t cap, double *__restrict__ T2,
-                const double *__restrict__ T, const double *__restrict__ Ci, int nx, int ny,
+    k_fixup_f64(void *fix, size_t cap, double *T2, const double *T, const double *Ci, int nx, int ny,
                 Coef c0) {
   __shared__ long long queue[8][64];
+  pdl_trigger();
+  pdl_wait();
   const FixList fl = fix_list(fix, cap);
   const unsigned count = (unsigned)min((size_t)*(volatile unsigned *)fl.count, cap);
   const W<double> w = make_w(c0, 0.0);
@@ -507,12 +512,12 @@ __global__ void __launch_bounds__(256)
   unsigned nque = 0u;  // warp-uniform
   unsigned segs = 0u, pts = 0u;
   auto stencil = [&](long long p, double *tn) {
-    tn[0] = __ldg(T + p - 1);
-    tn[1] = __ldg(T + p + 1);
-    tn[2] = __ldg(T + p - sy);
-    tn[3] = __ldg(T + p + sy);
-    tn[4] = __ldg(T + p - sz);
-    tn[5] = __ldg(T + p + sz);
+    tn[0] = T[p - 1];
+    tn[1] = T[p + 1];
+    tn[2] = T[p - sy];
+    tn[3] = T[p + sy];
+    tn[4] = T[p - sz];
+    tn[5] = T[p + sz];
   };
   // the FP64 cell for the first n queued points
   auto run_queue = [&](unsigned n) {
@@ -521,7 +526,7 @@ __global__ void __launch_bounds__(256)
       const long long p = que[lane];
       double tn[6];
       stencil(p, tn);
-      T2[p] = cell_f64(__ldg(T + p), tn[0], tn[1], tn[2], tn[3], tn[4], tn[5], __ldg(Ci + p), w);
+      T2[p] = cell_f64(T[p], tn[0], tn[1], tn[2], tn[3], tn[4], tn[5], Ci[p], w);
     }
     __syncwarp();
   };
@@ -536,7 +541,7 @@ __global__ void __launch_bounds__(256)
       if (on && in_bounds(p - sz, c0.npts) && in_bounds(p + sz, c0.npts)) {
         double tn[6];
         stencil(p, tn);
-        const double tc = __ldg(T + p), ci = __ldg(Ci + p);
+        const double tc = T[p], ci = Ci[p];
         unsigned long long nb[6];
 #pragma unroll
         for (int i = 0; i < 6; ++i) nb[i] = dbits(tn[i]);
@@ -650,15 +655,12 @@ cudaError_t launch_t(const TmaTile *tiles, int ntiles, void *T2, const void *T, 
   if (!ok) return cudaErrorInvalidValue;
   Coef cc = c;
   cc.npts = (long long)nx * ny * nzt;
-  k_stencil_tma<S, Shp::LPR, Shp::H, SWAP, MODE>
-      <<<ntiles, 32 * (Sh::CONSUMERS + 1), Sh::SMEM, s>>>(mT, mC, tiles, (S *)T2, nx, ny, cc,
-                                                          dev_err, fix.p, fix.cap);
-  cudaError_t e = cudaGetLastError();
-  if (e == cudaSuccess && is_emu(MODE)) {
-    k_fixup_f64<emu_groups(MODE)><<<kFixupBlocks, 256, 0, s>>>(
-        fix.p, fix.cap, (double *)T2, (const double *)T, (const double *)Ci, nx, ny, cc);
-    e = cudaGetLastError();
-  }
+  cudaError_t e = launch_pdl(pdl_on(cc.npts), k_stencil_tma<S, Shp::LPR, Shp::H, SWAP, MODE>, ntiles,
+                             32 * (Sh::CONSUMERS + 1), Sh::SMEM, s, mT, mC, tiles, (S *)T2, nx, ny,
+                             cc, dev_err, fix.p, fix.cap, TmaBatch());
+  if (e == cudaSuccess && is_emu(MODE))
+    e = launch_pdl(pdl_on(cc.npts), k_fixup_f64<emu_groups(MODE)>, kFixupBlocks, 256, 0, s, fix.p, fix.cap, (double *)T2,
+                   (const double *)T, (const double *)Ci, nx, ny, cc);
   return e;
 }
 
@@ -735,10 +737,9 @@ cudaError_t launch_batch_t(const TmaTile *tiles, int ntiles, void *T2, const Tma
   constexpr int MODE = sizeof(S) == 8 ? MODE_F64 : MODE_CELL;
   CUtensorMap none;
   std::memset(&none, 0, sizeof none);
-  k_stencil_tma<S, Shp::LPR, Shp::H, false, MODE, true>
-      <<<ntiles, 32 * (Sh::CONSUMERS + 1), Sh::SMEM, s>>>(none, none, tiles, (S *)T2, 0, 0,
-                                                          Coef(), dev_err, nullptr, 0, b);
-  return cudaGetLastError();
+  return launch_pdl(ntiles <= 4 * 152, k_stencil_tma<S, Shp::LPR, Shp::H, false, MODE, true>, ntiles,
+                    32 * (Sh::CONSUMERS + 1), Sh::SMEM, s, none, none, tiles, (S *)T2, 0, 0, Coef(),
+                    dev_err, nullptr, 0, b);
 }
 
 template <class S>
