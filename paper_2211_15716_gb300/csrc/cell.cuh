@@ -17,6 +17,7 @@
 #include <cuda_bf16.h>
 
 #include "igg_internal.h"
+#include "pair.cuh"
 
 namespace igg {
 namespace {
@@ -337,30 +338,7 @@ __device__ __forceinline__ bool emu_spread_d(double tc, const unsigned long long
 // row neighbour shares them, so the TMA kernel's pairs of points take both
 // from the first point of the pair.
 // ---------------------------------------------------------------------------
-// Pairs of FP32 numbers use the packed instructions. The sums below are
-// written so that no product feeds an addition (products are FMAs with a
-// zero addend, or folded into the FMA that uses them): the compiler may fuse
-// a packed multiply into a following packed addition, which would change the
-// rounding against the scalar form.
-__device__ __forceinline__ float vadd(float a, float b) { return __fadd_rn(a, b); }
-__device__ __forceinline__ float2 vadd(float2 a, float2 b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ float vneg(float a) { return -a; }
-__device__ __forceinline__ float2 vneg(float2 a) { return make_float2(-a.x, -a.y); }
-__device__ __forceinline__ float vfma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
-__device__ __forceinline__ float2 vfma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
-__device__ __forceinline__ float vset(float w, float) { return w; }
-__device__ __forceinline__ float2 vset(float w, float2) { return make_float2(w, w); }
-
 constexpr float kMagic = 12582912.0f;  // 1.5 * 2^23
-
-// error-free sum a + b = s + e (Knuth's two-sum), per lane
-template <class V>
-__device__ __forceinline__ V vtwo_sum(V a, V b, V &e) {
-  const V s = vadd(a, b);
-  const V bb = vadd(s, vneg(a));
-  e = vadd(vadd(a, vneg(vadd(s, vneg(bb)))), vadd(b, vneg(bb)));
-  return s;
-}
 
 // The centre's part of the fast-path test: sign and exponent field E in
 // [180, 2008] (hc: the centre's high word).

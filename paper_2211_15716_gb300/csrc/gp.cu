@@ -94,67 +94,80 @@ __device__ __forceinline__ FF gp_pair(double x) {
   return q;
 }
 
+// the pairs of two points
+__device__ __forceinline__ FF2 gp_pair2(double a, double b) {
+  const FF p = gp_pair(a), q = gp_pair(b);
+  return {make_float2(p.h, q.h), make_float2(p.l, q.l)};
+}
+
 // q = dt (V + g (u^2 + v^2)) in FP64 (uc, vc: u and v at the point)
 __device__ __forceinline__ double gp_q(double uc, double vc, double pot, const GpPairW &w) {
   return __dmul_rn(w.dt, __fma_rn(w.g, __fma_rn(uc, uc, __dmul_rn(vc, vc)), pot));
 }
 
-// q as a normalised pair from the pairs of u and v (NaN in h when a pair
-// is, or when the potential lies outside the pair range): error-free
-// squares and sum for rho, then g rho + V and dt (..) with FMA product
-// splits, about 2^-45 of dt (|V| + |g| rho)
-__device__ __forceinline__ FF gp_q_pair(const FF &u, const FF &v, double pot, const GpPairW &w) {
-  const float p1 = __fmul_rn(u.h, u.h);
-  float e1 = __fmaf_rn(u.h, u.h, -p1);
-  e1 = __fmaf_rn(__fadd_rn(u.h, u.h), u.l, e1);
-  const float p2 = __fmul_rn(v.h, v.h);
-  float e2 = __fmaf_rn(v.h, v.h, -p2);
-  e2 = __fmaf_rn(__fadd_rn(v.h, v.h), v.l, e2);
-  float t;
-  const float rs = pair_two_sum(p1, p2, t);
-  t = __fadd_rn(t, __fadd_rn(e1, e2));
-  const float a = __fmul_rn(w.gh, rs);
-  float ae = __fmaf_rn(w.gh, rs, -a);
-  ae = __fmaf_rn(w.gh, t, ae);
-  ae = __fmaf_rn(w.gl, rs, ae);
-  FF vp = pair_split(pot);
-  vp.h = pair_ok(pot, kGpWE) ? vp.h : __int_as_float(0x7FC00000);
-  float be;
-  const float b = pair_two_sum(a, vp.h, be);
-  be = __fadd_rn(be, __fadd_rn(ae, vp.l));
-  const float cq = __fmul_rn(w.dth, b);
-  float ce = __fmaf_rn(w.dth, b, -cq);
-  ce = __fmaf_rn(w.dth, be, ce);
-  ce = __fmaf_rn(w.dtl, b, ce);
-  FF q;
-  q.h = fast_two_sum(cq, ce, q.l);
+// q as a normalised pair from the pairs of u, v and the potential (NaN in h
+// when one of theirs is): error-free squares and sum for rho, then g rho + V
+// and dt (..) with FMA product splits, about 2^-45 of dt (|V| + |g| rho). One
+// point, or two as float2 (the same roundings).
+template <class F>
+__device__ __forceinline__ FFv<F> gp_q_pair(const FFv<F> &u, const FFv<F> &v, const FFv<F> &vp,
+                                            const GpPairW &w) {
+  const F zero = vset(0.f, F());
+  const F p1 = vfma(u.h, u.h, zero);
+  F e1 = vfma(u.h, u.h, vneg(p1));
+  e1 = vfma(vadd(u.h, u.h), u.l, e1);
+  const F p2 = vfma(v.h, v.h, zero);
+  F e2 = vfma(v.h, v.h, vneg(p2));
+  e2 = vfma(vadd(v.h, v.h), v.l, e2);
+  F t;
+  const F rs = vtwo_sum(p1, p2, t);
+  t = vadd(t, vadd(e1, e2));
+  const F gh = vset(w.gh, F()), dth = vset(w.dth, F());
+  const F a = vfma(gh, rs, zero);
+  F ae = vfma(gh, rs, vneg(a));
+  ae = vfma(gh, t, ae);
+  ae = vfma(vset(w.gl, F()), rs, ae);
+  F be;
+  const F b = vtwo_sum(a, vp.h, be);
+  be = vadd(be, vadd(ae, vp.l));
+  const F cq = vfma(dth, b, zero);
+  F ce = vfma(dth, b, vneg(cq));
+  ce = vfma(dth, be, ce);
+  ce = vfma(vset(w.dtl, F()), b, ce);
+  FFv<F> q;
+  q.h = vfast_two_sum(cq, ce, q.l);
   return q;
 }
 
 // the pair range of q: zero or |q| in [2^-36, 2^37) (from the leading part)
-__device__ __forceinline__ bool gp_q_ok(const FF &q) {
-  const unsigned b = __float_as_uint(q.h);
+__device__ __forceinline__ bool gp_q_ok(float qh) {
+  const unsigned b = __float_as_uint(qh);
   const unsigned e = (b >> 23) & 0xFFu;
   return e - (127u - kGpQE) <= 2u * kGpQE || (b << 1) == 0u;
 }
 
-// o + s h on the pair path from the pairs of o (op; o_ok: o in range) and
-// q; false: take gp_out_f64
-__device__ __forceinline__ bool gp_out_pair(const FF &op, bool o_ok, FF qp, const FF &wc,
-                                            const FF &wxm, const FF &wxp, const FF &wym,
-                                            const FF &wyp, const FF &wzm, const FF &wzp,
-                                            const GpPairW &w, double &res) {
-  const bool q_ok = gp_q_ok(qp);
-  qp.h *= w.s;
-  qp.l *= w.s;
-  float acc = op.h, err = op.l;
-  dot2_term(acc, err, w.kh[3], w.kl[3], wc.h, wc.l);
-  dot2_term(acc, err, qp.h, qp.l, wc.h, wc.l);
+// o + s h on the pair path as acc + err, from the pairs of o, q and w (one
+// point, or two as float2)
+template <int WHICH, class F>
+__device__ __forceinline__ void gp_sum_pair(const FFv<F> &op, const FFv<F> &qp, const FFv<F> &wc,
+                                            const FFv<F> &wxm, const FFv<F> &wxp,
+                                            const FFv<F> &wym, const FFv<F> &wyp,
+                                            const FFv<F> &wzm, const FFv<F> &wzp,
+                                            const GpPairW &w, F &acc, F &err) {
+  acc = op.h;
+  err = op.l;
+  dot2_term(acc, err, vset(w.kh[3], F()), vset(w.kl[3], F()), wc.h, wc.l);
+  dot2_term(acc, err, WHICH == 0 ? qp.h : vneg(qp.h), WHICH == 0 ? qp.l : vneg(qp.l), wc.h, wc.l);
   dot2_pair(acc, err, w.kh[0], w.kl[0], wxm, wxp);
   dot2_pair(acc, err, w.kh[1], w.kl[1], wym, wyp);
   dot2_pair(acc, err, w.kh[2], w.kl[2], wzm, wzp);
+}
+
+// the sum rounded to FP64; false: take gp_out_f64 (o_ok: o in range)
+__device__ __forceinline__ bool gp_out_pair(float acc, float err, bool o_ok, float qh,
+                                            const GpPairW &w, double &res) {
   res = __dadd_rn(f2d_finite(acc), f2d_finite(err));
-  return w.pair && o_ok && q_ok && acc == acc;
+  return w.pair && o_ok && gp_q_ok(qh) && acc == acc;
 }
 
 // o + s h in FP64
@@ -217,10 +230,13 @@ __global__ void __launch_bounds__(kGpX *kGpY)
       const double o = out[p], pot = Vs[p];
       const double xm = w[p - 1], xp = w[p + 1], ym = w[p - sy], yp = w[p + sy];
       const FF op = gp_pair(o), cp = gp_pair(wc);
-      const FF qp = WHICH == 0 ? gp_q_pair(op, cp, pot, pw) : gp_q_pair(cp, op, pot, pw);
+      const FF vp = gp_pair(pot);
+      const FF qp = WHICH == 0 ? gp_q_pair(op, cp, vp, pw) : gp_q_pair(cp, op, vp, pw);
+      float acc, err;
+      gp_sum_pair<WHICH>(op, qp, cp, gp_pair(xm), gp_pair(xp), gp_pair(ym), gp_pair(yp),
+                         gp_pair(wm), gp_pair(wp), pw, acc, err);
       double r;
-      const bool ok = gp_out_pair(op, pair_ok(o, kGpWE), qp, cp, gp_pair(xm), gp_pair(xp),
-                                  gp_pair(ym), gp_pair(yp), gp_pair(wm), gp_pair(wp), pw, r);
+      const bool ok = gp_out_pair(acc, err, pair_ok(o, kGpWE), qp.h, pw, r);
       if (__any_sync(0xffffffffu, !ok)) {
         if (!ok) {
           const double q = WHICH == 0 ? gp_q(o, wc, pot, pw) : gp_q(wc, o, pot, pw);
@@ -255,15 +271,21 @@ struct GpShape {
   static constexpr int V = 16 / (int)sizeof(S);          // points per lane
   static constexpr int W = 32 * V;                       // points per row
   static constexpr int BW = W + 2 * V;                   // w box width
-  static constexpr int H = 16;                           // rows per tile
+  // rows per tile and stages: FP64 8 and 4, three CTAs per SM; FP32 16 and 6, one.
+  // The FP64 launch is bound by instruction issue (255 instructions per point,
+  // 2.4 per clock at 15 warps per SM, the barrier of each plane its first
+  // stall): 2x2x2 x 256^3, four steps, with one CTA of 16 rows 10.79, two of 8
+  // (six stages) 11.29, three of 8 10.76 ms
+  static constexpr int H = sizeof(S) == 8 ? 8 : 16;
   static constexpr int BH = H + 2;
   static constexpr int WARPS = H;
-  static constexpr int NS = 6;                           // loads issued NS - 2 ahead
+  static constexpr int MINB = H == 8 ? 3 : 1;            // resident CTAs per SM
+  static constexpr int NS = H == 8 ? 4 : 6;                           // loads issued NS - 2 ahead
   static constexpr int FB = BW * BH * (int)sizeof(S);    // w box bytes
   static constexpr int FBA = (FB + 127) / 128 * 128;
   static constexpr int OB = W * H * (int)sizeof(S);      // o and V box bytes
   static constexpr int STAGE = FBA + 2 * OB;
-  static constexpr int VPL = BW * BH;                    // pair plane elements
+  static constexpr int VPL = BW * BH;                    // pair plane points
   static constexpr int VBA = PAIRS ? (3 * VPL * 8 + 127) / 128 * 128 : 0;
   static constexpr int SMEM = NS * STAGE + VBA + NS * 8 + 16;
   static constexpr int RING = 2 * (W + 2) + 2 * H;
@@ -280,17 +302,18 @@ __device__ __forceinline__ void gp_lds16(const void *p, Vec<S> &o) {
 // mW, mO, mV: tensor maps of the field read (w), the field written (o) and
 // the potential over [nsub * nz][ny][nx]; ncxy columns per subdomain
 template <class S, int WHICH>
-__global__ void __launch_bounds__(32 * GpShape<S>::WARPS, 1)
+__global__ void __launch_bounds__(32 * GpShape<S>::WARPS, GpShape<S>::MINB)
     k_gp_tma(const __grid_constant__ CUtensorMap mW, const __grid_constant__ CUtensorMap mO,
              const __grid_constant__ CUtensorMap mV, int nx, int ny, int nz, int ncx, int ncxy,
-             int ncol, S *__restrict__ out, const GpPairW pw, const int *__restrict__ nbr, int ox,
+             int ncol, S *out, const S *rd, const GpPairW pw, const int *__restrict__ nbr, int ox,
              int xsend, unsigned *__restrict__ dev_err) {
   using Sh = GpShape<S>;
   constexpr int V = Sh::V, W = Sh::W, BW = Sh::BW, H = Sh::H, NS = Sh::NS;
   constexpr unsigned NT = 32 * Sh::WARPS;
   extern __shared__ __align__(128) unsigned char smem[];
   const unsigned sbase = smem_u32(smem);
-  FF *planes = reinterpret_cast<FF *>(smem + NS * Sh::STAGE);
+  // FP64: pair planes, two neighbouring points of a row as h0 h1 l0 l1
+  float *planes = reinterpret_cast<float *>(smem + NS * Sh::STAGE);
   const unsigned full0 = sbase + NS * Sh::STAGE + Sh::VBA;
   volatile int *flags = reinterpret_cast<volatile int *>(smem + NS * Sh::STAGE + Sh::VBA + NS * 8);
 
@@ -358,8 +381,8 @@ __global__ void __launch_bounds__(32 * GpShape<S>::WARPS, 1)
   int k = 0, q = 0;
   bool stop = false;
   // own w of planes z-1, z, z+1 (FP64: also as pairs)
-  S tm[V], tc[V], tp[V];
-  FF pm[V], pc[V], pp[V];
+  S tm[V], tc[V], tp[V];  // (FP64: unused)
+  FF2 pm, pc, pp;
   while (!stop && sh.next(sg)) {
     int x0, r0, zoff;
     origin(sg.col, x0, r0, zoff);
@@ -402,25 +425,29 @@ __global__ void __launch_bounds__(32 * GpShape<S>::WARPS, 1)
       rb[j] = i < Sh::RING ? (yo + 1) * BW + xo + V : -1;
     }
     // own w of load kk (and, FP64, its pairs)
-    auto own = [&](int kk, S *t, FF *pr) {
+    auto own = [&](int kk, S *t, FF2 &pr) {
       Vec<S> a;
       gp_lds16<S>(wbox(kk) + ob, a);
+      if constexpr (Sh::PAIRS) {
+        pr = gp_pair2(a.v[0], a.v[1]);
+      } else {
 #pragma unroll
-      for (int i = 0; i < V; ++i) {
-        t[i] = a.v[i];
-        if constexpr (Sh::PAIRS) pr[i] = gp_pair(a.v[i]);
+        for (int i = 0; i < V; ++i) t[i] = a.v[i];
       }
     };
     // FP64: the pair plane of load kk (own pairs, then the ring)
-    auto form = [&](int kk, FF *pl, const FF *pr) {
+    auto form = [&](int kk, float *pl, const FF2 &pr) {
       if constexpr (Sh::PAIRS) {
-        uint4 w4;
-        memcpy(&w4, pr, 16);
-        *reinterpret_cast<uint4 *>(pl + ob) = w4;
+        *reinterpret_cast<float4 *>(pl + 2 * ob) = make_float4(pr.h.x, pr.h.y, pr.l.x, pr.l.y);
         const S *Wb = wbox(kk);
 #pragma unroll
         for (int j = 0; j < Sh::RPT; ++j)
-          if (rb[j] >= 0) pl[rb[j]] = gp_pair(Wb[rb[j]]);
+          if (rb[j] >= 0) {
+            const FF q = gp_pair(Wb[rb[j]]);
+            float *d = pl + 4 * (rb[j] >> 1) + (rb[j] & 1);
+            d[0] = q.h;
+            d[2] = q.l;
+          }
       }
     };
     bool good = wait_full(k);
@@ -429,7 +456,7 @@ __global__ void __launch_bounds__(32 * GpShape<S>::WARPS, 1)
       ++k;
       good = wait_full(k);
     }
-    FF *pl = planes + (q % 3) * Sh::VPL;
+    float *pl = planes + (q % 3) * 2 * Sh::VPL;
     if (good) {
       own(k, tc, pc);
       form(k, pl, pc);
@@ -441,12 +468,12 @@ __global__ void __launch_bounds__(32 * GpShape<S>::WARPS, 1)
     if (threadIdx.x == 0) issue_upto(k + NS - 2);
     int kc = k;
     ++k;
-    const FF *plm = pl;
+    const float *plm = pl;
     ++q;
     for (int m = sg.m0; m < sg.m1; ++m) {
       const int z = m + 1;
       good = wait_full(k);
-      FF *pln = planes + (q % 3) * Sh::VPL;
+      float *pln = planes + (q % 3) * 2 * Sh::VPL;
       if (good) {
         own(k, tp, pp);
         form(k, pln, pp);
@@ -460,42 +487,52 @@ __global__ void __launch_bounds__(32 * GpShape<S>::WARPS, 1)
       const S *Wb = wbox(kc);
       const S *Ob = reinterpret_cast<const S *>(stage(kc) + Sh::FBA) + oo;
       const S *Pb = reinterpret_cast<const S *>(stage(kc) + Sh::FBA + Sh::OB) + oo;
-      Vec<S> ov, pv, wym, wyp;
+      Vec<S> ov, pv;
       gp_lds16<S>(Ob, ov);
       gp_lds16<S>(Pb, pv);
-      gp_lds16<S>(Wb + ob - BW, wym);
-      gp_lds16<S>(Wb + ob + BW, wyp);
-      const S wl = Wb[ob - 1], wr = Wb[ob + V];
+      const long long p0 = zoff * sz + xs + (long long)nx * y + sz * z;
       S res[V];
       if constexpr (Sh::PAIRS) {
-        const FF fl = plm[ob - 1], fr = plm[ob + V];
-        bool bad = false;
-#pragma unroll
-        for (int i = 0; i < V; ++i) {
-          const FF op = gp_pair(ov.v[i]);
-          const FF qp = WHICH == 0 ? gp_q_pair(op, pc[i], pv.v[i], pw)
-                                   : gp_q_pair(pc[i], op, pv.v[i], pw);
-          const FF xm = i == 0 ? fl : pc[i - 1];
-          const FF xp = i == V - 1 ? fr : pc[i + 1];
-          const bool ok = gp_out_pair(op, pair_ok(ov.v[i], kGpWE), qp, pc[i], xm, xp,
-                                      plm[ob - BW + i], plm[ob + BW + i], pm[i], pp[i], pw,
-                                      res[i]);
-          bad = bad || (!ok && xyin[i]);
-          if (!ok) res[i] = __longlong_as_double(0x7FF8000000000000ll);  // marks the point
-        }
+        // (the plane's row pitch and ob are even: ob and ob +- BW start pairs)
+        auto two = [&](int o) {
+          const float4 a = *reinterpret_cast<const float4 *>(plm + 2 * o);
+          return FF2{make_float2(a.x, a.y), make_float2(a.z, a.w)};
+        };
+        const float *xl = plm + 2 * ob - 4, *xr = plm + 2 * ob + 4;
+        const FF2 xm = {make_float2(xl[1], pc.h.x), make_float2(xl[3], pc.l.x)};
+        const FF2 xp = {make_float2(pc.h.y, xr[0]), make_float2(pc.l.y, xr[2])};
+        const FF2 op = gp_pair2(ov.v[0], ov.v[1]), vp = gp_pair2(pv.v[0], pv.v[1]);
+        const FF2 qp = WHICH == 0 ? gp_q_pair(op, pc, vp, pw) : gp_q_pair(pc, op, vp, pw);
+        float2 acc, err;
+        gp_sum_pair<WHICH>(op, qp, pc, xm, xp, two(ob - BW), two(ob + BW), pm, pp, pw, acc, err);
+        const bool ok0 =
+            gp_out_pair(acc.x, err.x, pair_ok(ov.v[0], kGpWE), qp.h.x, pw, res[0]);
+        const bool ok1 =
+            gp_out_pair(acc.y, err.y, pair_ok(ov.v[1], kGpWE), qp.h.y, pw, res[1]);
+        const bool bad = (!ok0 && xyin[0]) || (!ok1 && xyin[1]);
+        // (a NaN marks the point)
+        if (!ok0) res[0] = __longlong_as_double(0x7FF8000000000000ll);
+        if (!ok1) res[1] = __longlong_as_double(0x7FF8000000000000ll);
         if (__any_sync(0xffffffffu, bad)) {
 #pragma unroll
           for (int i = 0; i < V; ++i) {
             if (res[i] != res[i]) {
-              const double xm = i == 0 ? wl : tc[i - 1];
-              const double xp = i == V - 1 ? wr : tc[i + 1];
-              const double q = WHICH == 0 ? gp_q(ov.v[i], tc[i], pv.v[i], pw)
-                                          : gp_q(tc[i], ov.v[i], pv.v[i], pw);
-              res[i] = gp_out_f64(ov.v[i], q, tc[i], xm, xp, wym.v[i], wyp.v[i], tm[i], tp[i], pw);
+              // (the field read is not written by this launch; planes z and
+              // z + 1 are in shared memory, z - 1 may have been overwritten)
+              const double *wc = reinterpret_cast<const double *>(Wb) + ob + i;
+              const double wzm = xyin[i] ? rd[p0 + i - sz] : 0.0;
+              const double wzp = reinterpret_cast<const double *>(wbox(k))[ob + i];
+              const double q = WHICH == 0 ? gp_q(ov.v[i], wc[0], pv.v[i], pw)
+                                          : gp_q(wc[0], ov.v[i], pv.v[i], pw);
+              res[i] = gp_out_f64(ov.v[i], q, wc[0], wc[-1], wc[1], wc[-BW], wc[BW], wzm, wzp, pw);
             }
           }
         }
       } else {
+        Vec<S> wym, wyp;
+        gp_lds16<S>(Wb + ob - BW, wym);
+        gp_lds16<S>(Wb + ob + BW, wyp);
+        const S wl = Wb[ob - 1], wr = Wb[ob + V];
 #pragma unroll
         for (int i = 0; i < V; ++i) {
           const S xm = i == 0 ? wl : tc[i - 1];
@@ -505,7 +542,6 @@ __global__ void __launch_bounds__(32 * GpShape<S>::WARPS, 1)
                               tp[i], pw, WHICH);
         }
       }
-      const long long p0 = zoff * sz + xs + (long long)nx * y + sz * z;
       bool all_in = true;
 #pragma unroll
       for (int i = 0; i < V; ++i) all_in = all_in && xyin[i];
@@ -532,13 +568,15 @@ __global__ void __launch_bounds__(32 * GpShape<S>::WARPS, 1)
       ++k;
       plm = pln;
       ++q;
+      if constexpr (!Sh::PAIRS) {
 #pragma unroll
-      for (int i = 0; i < V; ++i) {
-        tm[i] = tc[i];
-        tc[i] = tp[i];
-        pm[i] = pc[i];
-        pc[i] = pp[i];
+        for (int i = 0; i < V; ++i) {
+          tm[i] = tc[i];
+          tc[i] = tp[i];
+        }
       }
+      pm = pc;
+      pc = pp;
     }
   }
   if (threadIdx.x == 0) flags[0] = issued;
@@ -588,7 +626,7 @@ cudaError_t launch_tma(int nsub, int nx, int ny, int nz, void *u, void *v, const
   const long long U = ncol * (nz - 2);
   const long long G = std::min<long long>((long long)per_sm * sms, std::max<long long>(1, U / 4));
   return launch_pdl(pdl_on((long long)nsub * nx * ny * nz), k_gp_tma<S, WHICH>, (unsigned)G, 32 * Sh::WARPS, Sh::SMEM, s, mW, mO, mV, nx,
-                    ny, nz, ncx, ncx * ncy, (int)ncol, (S *)o, make_gp_w(c, WHICH), c.nbr, c.ox,
+                    ny, nz, ncx, ncx * ncy, (int)ncol, (S *)o, (const S *)w, make_gp_w(c, WHICH), c.nbr, c.ox,
                     c.xsend, dev_err);
 }
 

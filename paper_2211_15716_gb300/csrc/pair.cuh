@@ -12,10 +12,37 @@
 namespace igg {
 namespace {
 
-// float pair h + l
-struct FF {
-  float h, l;
+// FP32 arithmetic on one number or, as float2, on two points at once (packed
+// instructions: half the issue slots). The sums below are
+// written so that no product feeds an addition (products are FMAs with a
+// zero addend, or folded into the FMA that uses them): the compiler may fuse
+// a packed multiply into a following packed addition, which would change the
+// rounding against the scalar form.
+__device__ __forceinline__ float vadd(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float2 vadd(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float vneg(float a) { return -a; }
+__device__ __forceinline__ float2 vneg(float2 a) { return make_float2(-a.x, -a.y); }
+__device__ __forceinline__ float vfma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ float2 vfma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float vset(float w, float) { return w; }
+__device__ __forceinline__ float2 vset(float w, float2) { return make_float2(w, w); }
+
+// error-free sum a + b = s + e (Knuth's two-sum), per lane
+template <class V>
+__device__ __forceinline__ V vtwo_sum(V a, V b, V &e) {
+  const V s = vadd(a, b);
+  const V bb = vadd(s, vneg(a));
+  e = vadd(vadd(a, vneg(vadd(s, vneg(bb)))), vadd(b, vneg(bb)));
+  return s;
+}
+
+// float pair h + l (F = float2: of two points)
+template <class F>
+struct FFv {
+  F h, l;
 };
+using FF = FFv<float>;
+using FF2 = FFv<float2>;
 
 // True when x is zero or its exponent field lies in [1023 - r, 1023 + r].
 // Radii of at most 127 keep that inside pair_split's range [949, 1150].
@@ -68,40 +95,42 @@ __device__ __forceinline__ double f2d_finite(float f) {
   return __hiloint2double((int)hi, z ? 0 : (int)(b << 29));
 }
 
-// error-free sum of two floats: a + b = s + e exactly
-__device__ __forceinline__ float pair_two_sum(float a, float b, float &e) {
-  const float s = __fadd_rn(a, b);
-  const float bb = __fsub_rn(s, a);
-  e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
+// error-free sum when |a| >= |b| or a == 0 (Dekker): a + b = s + e exactly
+template <class F>
+__device__ __forceinline__ F vfast_two_sum(F a, F b, F &e) {
+  const F s = vadd(a, b);
+  e = vadd(b, vneg(vadd(s, vneg(a))));
   return s;
 }
 
 // acc + err += w * v (w, v pairs): error-free leading product and sum, the
 // small parts into err
-__device__ __forceinline__ void dot2_term(float &acc, float &err, float wh, float wl, float vh,
-                                          float vl) {
-  const float p = __fmul_rn(wh, vh);
-  float q = __fmaf_rn(wh, vh, -p);
-  q = __fmaf_rn(wh, vl, q);
-  q = __fmaf_rn(wl, vh, q);
-  float e;
-  acc = pair_two_sum(acc, p, e);
-  err = __fadd_rn(err, __fadd_rn(e, q));
+template <class F>
+__device__ __forceinline__ void dot2_term(F &acc, F &err, F wh, F wl, F vh, F vl) {
+  const F p = vfma(wh, vh, vset(0.f, F()));
+  F q = vfma(wh, vh, vneg(p));
+  q = vfma(wh, vl, q);
+  q = vfma(wl, vh, q);
+  F e;
+  acc = vtwo_sum(acc, p, e);
+  err = vadd(err, vadd(e, q));
 }
 
 // acc + err += w * (a + b) for the neighbour pair (a, b)
-__device__ __forceinline__ void dot2_pair(float &acc, float &err, float wh, float wl, const FF &a,
-                                          const FF &b) {
-  float t;
-  const float s = pair_two_sum(a.h, b.h, t);
-  t = __fadd_rn(t, __fadd_rn(a.l, b.l));
-  const float p = __fmul_rn(wh, s);
-  float q = __fmaf_rn(wh, s, -p);
-  q = __fmaf_rn(wh, t, q);
-  q = __fmaf_rn(wl, s, q);
-  float e;
-  acc = pair_two_sum(acc, p, e);
-  err = __fadd_rn(err, __fadd_rn(e, q));
+template <class F>
+__device__ __forceinline__ void dot2_pair(F &acc, F &err, float wh, float wl, const FFv<F> &a,
+                                          const FFv<F> &b) {
+  F t;
+  const F s = vtwo_sum(a.h, b.h, t);
+  t = vadd(t, vadd(a.l, b.l));
+  const F h = vset(wh, F());
+  const F p = vfma(h, s, vset(0.f, F()));
+  F q = vfma(h, s, vneg(p));
+  q = vfma(h, t, q);
+  q = vfma(vset(wl, F()), s, q);
+  F e;
+  acc = vtwo_sum(acc, p, e);
+  err = vadd(err, vadd(e, q));
 }
 
 }  // namespace
