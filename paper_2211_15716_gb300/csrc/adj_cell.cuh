@@ -58,19 +58,24 @@ __device__ __forceinline__ FF pair_ci(double ci) {
   return b;
 }
 
-// v of one point for FP64 fields as a normalised pair from the pairs of lam
-// (pair_lam) and Ci (pair_ci); (0, 0) off the inner points; NaN in h when
-// either pair holds one (a value outside the pair range).
+// v for FP64 fields as a normalised pair from the pairs of lam (pair_lam) and
+// Ci (pair_ci); NaN in h when either pair holds one (a value outside the pair
+// range). One point, or two as float2 (the same roundings). The caller sets
+// (0, 0) off the inner points.
+template <class F>
+__device__ __forceinline__ FFv<F> adj_v_prod(const FFv<F> &a, const FFv<F> &b) {
+  const F p = vfma(a.h, b.h, vset(0.f, F()));
+  F e = vfma(a.h, b.h, vneg(p));
+  e = vfma(a.h, b.l, e);
+  e = vfma(a.l, b.h, e);
+  e = vfma(a.l, b.l, e);
+  FFv<F> v;
+  v.h = vfast_two_sum(p, e, v.l);
+  return v;
+}
+
 __device__ __forceinline__ FF adj_v_pairs(const FF &a, const FF &b, bool inner) {
-  const float p = __fmul_rn(a.h, b.h);
-  float e = __fmaf_rn(a.h, b.h, -p);
-  e = __fmaf_rn(a.h, b.l, e);
-  e = __fmaf_rn(a.l, b.h, e);
-  e = __fmaf_rn(a.l, b.l, e);
-  FF v;
-  float q;
-  v.h = fast_two_sum(p, e, q);
-  v.l = q;
+  FF v = adj_v_prod(a, b);
   v.h = inner ? v.h : 0.f;
   v.l = inner ? v.l : 0.f;
   return v;
@@ -110,18 +115,24 @@ __device__ __forceinline__ AdjW make_adj_w(const Coef &c) {
   return a;
 }
 
-// lam_out of one point on the pair path from lam as a pair (pair_lam);
-// false when the point must take the FP64 sum (a value outside the pair
-// ranges: a NaN reaches acc; or weights outside theirs).
-__device__ __forceinline__ bool adj_out_pair(const FF &lq, const FF &vc, const FF &vxm,
-                                             const FF &vxp, const FF &vym, const FF &vyp,
-                                             const FF &vzm, const FF &vzp, const AdjW &a,
-                                             double &out) {
-  float acc = lq.h, err = lq.l;
-  dot2_term(acc, err, a.wh[3], a.wl[3], vc.h, vc.l);
+// lam_out on the pair path as acc + err from lam as a pair (pair_lam): one
+// point, or two as float2
+template <class F>
+__device__ __forceinline__ void adj_sum_pair(const FFv<F> &lq, const FFv<F> &vc, const FFv<F> &vxm,
+                                             const FFv<F> &vxp, const FFv<F> &vym,
+                                             const FFv<F> &vyp, const FFv<F> &vzm,
+                                             const FFv<F> &vzp, const AdjW &a, F &acc, F &err) {
+  acc = lq.h;
+  err = lq.l;
+  dot2_term(acc, err, vset(a.wh[3], F()), vset(a.wl[3], F()), vc.h, vc.l);
   dot2_pair(acc, err, a.wh[0], a.wl[0], vxm, vxp);
   dot2_pair(acc, err, a.wh[1], a.wl[1], vym, vyp);
   dot2_pair(acc, err, a.wh[2], a.wl[2], vzm, vzp);
+}
+
+// the sum rounded to FP64; false when the point must take the FP64 sum (a
+// value outside the pair ranges: a NaN reaches acc; or weights outside theirs)
+__device__ __forceinline__ bool adj_out_pair(float acc, float err, const AdjW &a, double &out) {
   // a finite acc bounds err: both widen exactly (f2d_finite)
   out = __dadd_rn(f2d_finite(acc), f2d_finite(err));
   return a.pair && acc == acc;
@@ -174,6 +185,11 @@ __device__ __forceinline__ float adj_lap32(float c, float xm, float xp, float ym
 // (emu_spread_d); other stencils take the FP64 sum. The second and third
 // forms are reached only by warps with a point that needs them (branches on
 // warp votes). Every lane of the warp calls it.
+// NG: the weight groups where the kernel is compiled for them, 0: from w. (As a
+// branch on w inside the kernel the three forms were merged into predicated
+// code, two FP64 FMAs of each issued for every point: misfit gradient
+// at 256^3, 48 steps, 21.8 to 21.4 ms)
+template <int NG>
 __device__ __forceinline__ double gci_add(double g, bool inner, double la, double t, double xm,
                                           double xp, double ym, double yp, double zm, double zp,
                                           const W<double> &w) {
@@ -187,7 +203,8 @@ __device__ __forceinline__ double gci_add(double g, bool inner, double la, doubl
   }
   const bool ok = emu_fast_ok(dhi(t), hn);
   double r = g;
-  if (w.ng == 1) r = emu_apply(g, la, emu_lap<1>(t, nb, w));
+  if constexpr (NG > 0) r = emu_apply(g, la, emu_lap<NG>(t, nb, w));
+  else if (w.ng == 1) r = emu_apply(g, la, emu_lap<1>(t, nb, w));
   else if (w.ng == 2) r = emu_apply(g, la, emu_lap<2>(t, nb, w));
   else r = emu_apply(g, la, emu_lap<3>(t, nb, w));
   if (!__all_sync(0xffffffffu, ok || !inner)) {
@@ -195,7 +212,8 @@ __device__ __forceinline__ double gci_add(double g, bool inner, double la, doubl
     unsigned sh;
     const bool ok2 = emu_spread_d(t, nb, D, sh);
     if (inner && !ok && ok2) {
-      if (w.ng == 1) r = emu_apply(g, la, emu_lap_d<1>(D, sh, w));
+      if constexpr (NG > 0) r = emu_apply(g, la, emu_lap_d<NG>(D, sh, w));
+      else if (w.ng == 1) r = emu_apply(g, la, emu_lap_d<1>(D, sh, w));
       else if (w.ng == 2) r = emu_apply(g, la, emu_lap_d<2>(D, sh, w));
       else r = emu_apply(g, la, emu_lap_d<3>(D, sh, w));
     }
@@ -206,6 +224,7 @@ __device__ __forceinline__ double gci_add(double g, bool inner, double la, doubl
   }
   return inner ? r : g;
 }
+template <int NG>
 __device__ __forceinline__ double gci_add(double g, bool inner, float la, float t, float xm,
                                           float xp, float ym, float yp, float zm, float zp,
                                           const W<float> &w) {
@@ -233,7 +252,9 @@ struct AdjOps<double> {
                                              const FF &vxp, const FF &vym, const FF &vyp,
                                              const FF &vzm, const FF &vzp, const AdjW &a,
                                              double &o) {
-    return adj_out_pair(lq, vc, vxm, vxp, vym, vyp, vzm, vzp, a, o);
+    float acc, err;
+    adj_sum_pair(lq, vc, vxm, vxp, vym, vyp, vzm, vzp, a, acc, err);
+    return adj_out_pair(acc, err, a, o);
   }
   static __device__ __forceinline__ const W<double> &lapw(const AdjW &a) { return a.w; }
 };

@@ -127,7 +127,7 @@ __global__ void __launch_bounds__(kAdjX *kAdjY)
     if (own) lam_out[p] = out;
     const bool inner = own && in_xy && z > 0 && z < nz - 1;
     const double g = inner ? gCi[p] : 0.0;
-    const double gn = gci_add(g, inner, la, tc, ts[b][ty + 1][tx], ts[b][ty + 1][tx + 2],
+    const double gn = gci_add<0>(g, inner, la, tc, ts[b][ty + 1][tx], ts[b][ty + 1][tx + 2],
                               ts[b][ty][tx + 1], ts[b][ty + 2][tx + 1], tm, tp, Ops::lapw(aw));
     if (inner) gCi[p] = gn;
     vm = vc;

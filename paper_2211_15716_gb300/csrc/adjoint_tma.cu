@@ -71,6 +71,25 @@ struct AdjShape {
   static_assert(NS >= 4, "issue rule needs two loads ahead");
 };
 
+// The values a lane holds of one plane: FP64 two points as pairs (float2
+// arithmetic, half the issue slots of one point at a time: misfit gradient at
+// 256^3, 48 steps, 21.4 to 21.0 ms), FP32 four points.
+template <class S>
+struct AdjVec;
+template <>
+struct AdjVec<double> {
+  FF2 p;
+};
+template <>
+struct AdjVec<float> {
+  float p[4];
+};
+// v planes in shared memory: FP64 as h0 h1 l0 l1 for two neighbouring points
+__device__ __forceinline__ FF2 ld_pair2(const float *pl, int o) {
+  const float4 a = *reinterpret_cast<const float4 *>(pl + 2 * o);
+  return {make_float2(a.x, a.y), make_float2(a.z, a.w)};
+}
+
 template <class S>
 __device__ __forceinline__ void lds16(const void *p, Vec<S> &o) {
   unpack(*reinterpret_cast<const uint4 *>(p), o);
@@ -79,12 +98,14 @@ __device__ __forceinline__ void lds16(const void *p, Vec<S> &o) {
 // CIP (FP64 fields): the Ci box holds Ci as pairs (pair_ci, formed once per
 // run by k_pair_ci) instead of the FP64 values; the FP64 sum then reads Ci
 // from memory.
-template <class S, bool CIP>
+// NG: weight groups of gCi's Laplacian (FP64 fields; FP32: 0)
+template <class S, bool CIP, int NG>
 __global__ void __launch_bounds__(32 * AdjShape<S>::WARPS, AdjShape<S>::MINB)
     k_adjoint_tma(const __grid_constant__ CUtensorMap mL, const __grid_constant__ CUtensorMap mC,
                   const __grid_constant__ CUtensorMap mT, const __grid_constant__ CUtensorMap mG,
                   int nx, int ny, int nz, int ncx, int ncxy, int ncol, S *__restrict__ lam_out,
-                  const S *lam_in, const S *Ci, double *__restrict__ gCi, Coef c, unsigned *__restrict__ dev_err) {
+                  const S *lam_in, const S *Ci, double *__restrict__ gCi, Coef c,
+                  unsigned *__restrict__ dev_err) {
   using Sh = AdjShape<S>;
   using Ops = AdjOps<S>;
   using VT = typename Sh::VT;
@@ -93,7 +114,9 @@ __global__ void __launch_bounds__(32 * AdjShape<S>::WARPS, AdjShape<S>::MINB)
   constexpr unsigned NT = 32 * Sh::WARPS;
   extern __shared__ __align__(128) unsigned char smem[];
   const unsigned sbase = smem_u32(smem);
-  VT *vbuf = reinterpret_cast<VT *>(smem + NS * Sh::STAGE);
+  constexpr bool PAIRS = sizeof(S) == 8;
+  constexpr int VPF = Sh::VPL * (int)sizeof(VT) / 4;  // floats of a v plane
+  float *vbuf = reinterpret_cast<float *>(smem + NS * Sh::STAGE);
   const unsigned full0 = sbase + NS * Sh::STAGE + Sh::VBA;
   volatile int *flags = reinterpret_cast<volatile int *>(smem + NS * Sh::STAGE + Sh::VBA + NS * 8);
   // flags[0]: loads issued
@@ -169,8 +192,8 @@ __global__ void __launch_bounds__(32 * AdjShape<S>::WARPS, AdjShape<S>::MINB)
   // own values of planes m-1, m, m+1: lam (m, m+1: value and the sum's
   // start), T, v
   S lc[V], lp[V], tm[V], tc[V], tp[V];
-  LT qc[V], qp[V];
-  VT vm[V], vc[V], vp[V];
+  AdjVec<S> qc, qp;  // (FP32: unused, lc and lp)
+  AdjVec<S> vm, vc, vp;
   while (!stop && sh.next(sg)) {
     int x0, r0, zoff;
     origin(sg.col, x0, r0, zoff);
@@ -200,7 +223,7 @@ __global__ void __launch_bounds__(32 * AdjShape<S>::WARPS, AdjShape<S>::MINB)
       rxy[j] = xx >= 1 && xx <= nx - 2 && yy >= 1 && yy <= ny - 2;
     }
     // own values of plane p from load kk
-    auto own = [&](int kk, int p, S *l, LT *lq, S *t, VT *v) {
+    auto own = [&](int kk, int p, S *l, AdjVec<S> &lq, S *t, AdjVec<S> &v) {
       Vec<S> a, b, d;
       lds16<S>(box(kk, 0) + ob, a);
       lds16<S>(box(kk, 1) + ob, b);
@@ -208,46 +231,63 @@ __global__ void __launch_bounds__(32 * AdjShape<S>::WARPS, AdjShape<S>::MINB)
       const bool zi = zin(p);
 #pragma unroll
       for (int i = 0; i < V; ++i) {
-        const LT qq = Ops::lam(a.v[i]);
-        if (l) l[i] = a.v[i];
-        if (lq) lq[i] = qq;
+        l[i] = a.v[i];
         t[i] = d.v[i];
+      }
+      if constexpr (PAIRS) {
+        const FF q0 = pair_lam(a.v[0]), q1 = pair_lam(a.v[1]);
+        FF c0, c1;
         if constexpr (CIP) {
-          FF cp;
-          memcpy(&cp, &b.v[i], 8);
-          v[i] = adj_v_pairs(qq, cp, xyin[i] && zi);
+          memcpy(&c0, &b.v[0], 8);
+          memcpy(&c1, &b.v[1], 8);
         } else {
-          v[i] = Ops::v(qq, b.v[i], xyin[i] && zi);
+          c0 = pair_ci(b.v[0]);
+          c1 = pair_ci(b.v[1]);
         }
+        lq.p = {make_float2(q0.h, q1.h), make_float2(q0.l, q1.l)};
+        v.p = adj_v_prod(lq.p, FF2{make_float2(c0.h, c1.h), make_float2(c0.l, c1.l)});
+        if (!(xyin[0] && zi)) v.p.h.x = v.p.l.x = 0.f;
+        if (!(xyin[1] && zi)) v.p.h.y = v.p.l.y = 0.f;
+      } else {
+#pragma unroll
+        for (int i = 0; i < V; ++i) v.p[i] = Ops::v(a.v[i], b.v[i], xyin[i] && zi);
       }
     };
     // the v plane of plane p from load kk: own values v, the ring from the boxes
-    auto form = [&](int kk, int p, VT *vb, const VT *v) {
-      uint4 w4;
+    auto form = [&](int kk, int p, float *vb, const AdjVec<S> &v) {
       static_assert(sizeof(VT) * V == 16, "one 16-byte vector of v per lane");
-      memcpy(&w4, v, 16);
-      *reinterpret_cast<uint4 *>(vb + ob) = w4;
+      if constexpr (PAIRS)
+        *reinterpret_cast<float4 *>(vb + 2 * ob) =
+            make_float4(v.p.h.x, v.p.h.y, v.p.l.x, v.p.l.y);
+      else
+        *reinterpret_cast<float4 *>(vb + ob) = make_float4(v.p[0], v.p[1], v.p[2], v.p[3]);
       const S *L = box(kk, 0), *C = box(kk, 1);
       const bool zi = zin(p);
 #pragma unroll
       for (int j = 0; j < Sh::RPT; ++j) {
         if (rb[j] < 0) continue;
-        if constexpr (CIP) {
-          vb[rb[j]] = adj_v_pairs(Ops::lam(L[rb[j]]), reinterpret_cast<const FF *>(C)[rb[j]],
-                                  rxy[j] && zi);
+        VT q;
+        if constexpr (CIP)
+          q = adj_v_pairs(Ops::lam(L[rb[j]]), reinterpret_cast<const FF *>(C)[rb[j]], rxy[j] && zi);
+        else
+          q = Ops::v(Ops::lam(L[rb[j]]), C[rb[j]], rxy[j] && zi);
+        if constexpr (PAIRS) {
+          float *d = vb + 4 * (rb[j] >> 1) + (rb[j] & 1);
+          d[0] = q.h;
+          d[2] = q.l;
         } else {
-          vb[rb[j]] = Ops::v(Ops::lam(L[rb[j]]), C[rb[j]], rxy[j] && zi);
+          vb[rb[j]] = q;
         }
       }
     };
     // load of plane m0 - 1 (own values), then of plane m0 (own values, v plane)
     bool good = wait_full(k);
     if (good) {
-      own(k, sg.m0 - 1, nullptr, nullptr, tm, vm);
+      own(k, sg.m0 - 1, lc, qc, tm, vm);
       ++k;
       good = wait_full(k);
     }
-    VT *vb = vbuf + (q % 3) * Sh::VPL;
+    float *vb = vbuf + (q % 3) * VPF;
     if (good) {
       own(k, sg.m0, lc, qc, tc, vc);
       form(k, sg.m0, vb, vc);
@@ -261,12 +301,12 @@ __global__ void __launch_bounds__(32 * AdjShape<S>::WARPS, AdjShape<S>::MINB)
     if (threadIdx.x == 0) issue_upto(k + NS - 2);
     int kc = k;  // load of plane m
     ++k;
-    const VT *vbm = vb;
+    const float *vbm = vb;
     ++q;
     for (int m = sg.m0; m < sg.m1; ++m) {
       // plane m + 1: own values and v plane
       good = wait_full(k);
-      VT *vbn = vbuf + (q % 3) * Sh::VPL;
+      float *vbn = vbuf + (q % 3) * VPF;
       if (good) {
         own(k, m + 1, lp, qp, tp, vp);
         form(k, m + 1, vbn, vp);
@@ -280,17 +320,29 @@ __global__ void __launch_bounds__(32 * AdjShape<S>::WARPS, AdjShape<S>::MINB)
       const S *L = box(kc, 0), *C = box(kc, 1), *T = box(kc, 2);
       const double *G =
           reinterpret_cast<const double *>(stage(kc) + 3 * Sh::FBA) + r * W + lane * V;
-      const VT vl = vbm[ob - 1], vr = vbm[ob + V];
       S out[V];
       bool okp[V];
       bool any_bad = false;
+      if constexpr (PAIRS) {
+        const float *xl = vbm + 2 * ob - 4, *xr = vbm + 2 * ob + 4;
+        const FF2 &v = vc.p;
+        const FF2 xm = {make_float2(xl[1], v.h.x), make_float2(xl[3], v.l.x)};
+        const FF2 xp = {make_float2(v.h.y, xr[0]), make_float2(v.l.y, xr[2])};
+        float2 acc, err;
+        adj_sum_pair(qc.p, v, xm, xp, ld_pair2(vbm, ob - BW), ld_pair2(vbm, ob + BW), vm.p, vp.p, aw,
+                     acc, err);
+        okp[0] = adj_out_pair(acc.x, err.x, aw, out[0]);
+        okp[1] = adj_out_pair(acc.y, err.y, aw, out[1]);
+        any_bad = !okp[0] || !okp[1];
+      } else {
+        const float vl = vbm[ob - 1], vr = vbm[ob + V];
+        const float4 ym = *reinterpret_cast<const float4 *>(vbm + ob - BW);
+        const float4 yp = *reinterpret_cast<const float4 *>(vbm + ob + BW);
+        const float yma[4] = {ym.x, ym.y, ym.z, ym.w}, ypa[4] = {yp.x, yp.y, yp.z, yp.w};
 #pragma unroll
-      for (int i = 0; i < V; ++i) {
-        const VT xm = i == 0 ? vl : vc[i - 1];
-        const VT xp = i == V - 1 ? vr : vc[i + 1];
-        okp[i] = Ops::out(qc[i], vc[i], xm, xp, vbm[ob - BW + i], vbm[ob + BW + i], vm[i], vp[i],
-                          aw, out[i]);
-        any_bad = any_bad || !okp[i];
+        for (int i = 0; i < V; ++i)
+          Ops::out(lc[i], vc.p[i], i == 0 ? vl : vc.p[i - 1], i == V - 1 ? vr : vc.p[i + 1], yma[i],
+                   ypa[i], vm.p[i], vp.p[i], aw, out[i]);
       }
       if constexpr (sizeof(S) == 8) {
         // points outside the pair path's ranges: the FP64 sum, its v from
@@ -354,7 +406,7 @@ __global__ void __launch_bounds__(32 * AdjShape<S>::WARPS, AdjShape<S>::MINB)
         all_in = all_in && inn;
         const S xm = i == 0 ? tl : tc[i - 1];
         const S xp = i == V - 1 ? tr : tc[i + 1];
-        gn[i] = gci_add(G[i], inn, lc[i], tc[i], xm, xp, tym.v[i], typ.v[i], tm[i], tp[i],
+        gn[i] = gci_add<NG>(G[i], inn, lc[i], tc[i], xm, xp, tym.v[i], typ.v[i], tm[i], tp[i],
                         Ops::lapw(aw));
       }
       double *gd = gCi + p0;
@@ -374,12 +426,12 @@ __global__ void __launch_bounds__(32 * AdjShape<S>::WARPS, AdjShape<S>::MINB)
 #pragma unroll
       for (int i = 0; i < V; ++i) {
         lc[i] = lp[i];
-        qc[i] = qp[i];
         tm[i] = tc[i];
         tc[i] = tp[i];
-        vm[i] = vc[i];
-        vc[i] = vp[i];
       }
+      qc = qp;
+      vm = vc;
+      vc = vp;
     }
   }
   if (threadIdx.x == 0) flags[0] = issued;
@@ -397,21 +449,21 @@ __global__ void __launch_bounds__(32 * AdjShape<S>::WARPS, AdjShape<S>::MINB)
   }
 }
 
-template <class S, bool CIP>
+template <class S, bool CIP, int NG>
 cudaError_t prepare_adj_t(int *ctas_per_sm) {
   using Sh = AdjShape<S>;
   static cudaError_t done = cudaErrorNotReady;
   static std::mutex mu;
   std::lock_guard<std::mutex> lk(mu);
   if (done == cudaErrorNotReady)
-    done = cudaFuncSetAttribute(k_adjoint_tma<S, CIP>,
+    done = cudaFuncSetAttribute(k_adjoint_tma<S, CIP, NG>,
                                 cudaFuncAttributeMaxDynamicSharedMemorySize, Sh::SMEM);
   if (done != cudaSuccess) return done;
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas_per_sm, k_adjoint_tma<S, CIP>,
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas_per_sm, k_adjoint_tma<S, CIP, NG>,
                                                        32 * Sh::WARPS, Sh::SMEM);
 }
 
-template <class S, bool CIP>
+template <class S, bool CIP, int NG>
 cudaError_t launch_adj_t(int nsub, int nx, int ny, int nz, void *lam_out, const void *lam_in, const void *Tn,
                          const void *Ci, const void *ci_box, double *gCi, const Coef &c,
                          unsigned *dev_err, cudaStream_t s) {
@@ -425,7 +477,7 @@ cudaError_t launch_adj_t(int nsub, int nx, int ny, int nz, void *lam_out, const 
       !encode<double>(&mG, gCi, nx, ny, nzt, Sh::W, Sh::H, 1))
     return cudaErrorInvalidValue;
   int per_sm = 0, dev = 0, sms = 0;
-  cudaError_t e = prepare_adj_t<S, CIP>(&per_sm);
+  cudaError_t e = prepare_adj_t<S, CIP, NG>(&per_sm);
   if (e == cudaSuccess) e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
@@ -436,7 +488,7 @@ cudaError_t launch_adj_t(int nsub, int nx, int ny, int nz, void *lam_out, const 
   const long long U = ncol * nz;
   // every CTA gets at least a few planes; at most the resident CTAs
   const long long G = std::min<long long>((long long)per_sm * sms, std::max<long long>(1, U / 4));
-  return launch_pdl(pdl_on((long long)nsub * nx * ny * nz), k_adjoint_tma<S, CIP>, (unsigned)G, 32 * Sh::WARPS, Sh::SMEM, s, mL, mC, mT, mG,
+  return launch_pdl(pdl_on((long long)nsub * nx * ny * nz), k_adjoint_tma<S, CIP, NG>, (unsigned)G, 32 * Sh::WARPS, Sh::SMEM, s, mL, mC, mT, mG,
                     nx, ny, nz, ncx, ncx * ncy, (int)ncol, (S *)lam_out, (const S *)lam_in,
                     (const S *)Ci, gCi, c, dev_err);
 }
@@ -469,15 +521,20 @@ cudaError_t launch_adjoint_tma(igg_dtype dt, int nsub, int nx, int ny, int nz, v
                                const Coef &c, unsigned *dev_err, cudaStream_t s,
                                const void *ci_pairs) {
   switch (dt) {
-    case IGG_F64:
-      if (ci_pairs)
-        return launch_adj_t<double, true>(nsub, nx, ny, nz, lam_out, lam_in, Tn, Ci, ci_pairs, gCi, c,
-                                          dev_err, s);
-      return launch_adj_t<double, false>(nsub, nx, ny, nz, lam_out, lam_in, Tn, Ci, Ci, gCi, c,
-                                         dev_err, s);
+    case IGG_F64: {
+      const int ng = weight_groups(c.wx, c.wy, c.wz);
+      const void *box = ci_pairs ? ci_pairs : Ci;
+      auto f = ci_pairs ? (ng == 1   ? launch_adj_t<double, true, 1>
+                           : ng == 2 ? launch_adj_t<double, true, 2>
+                                     : launch_adj_t<double, true, 3>)
+                        : (ng == 1   ? launch_adj_t<double, false, 1>
+                           : ng == 2 ? launch_adj_t<double, false, 2>
+                                     : launch_adj_t<double, false, 3>);
+      return f(nsub, nx, ny, nz, lam_out, lam_in, Tn, Ci, box, gCi, c, dev_err, s);
+    }
     case IGG_F32:
-      return launch_adj_t<float, false>(nsub, nx, ny, nz, lam_out, lam_in, Tn, Ci, Ci, gCi, c,
-                                        dev_err, s);
+      return launch_adj_t<float, false, 0>(nsub, nx, ny, nz, lam_out, lam_in, Tn, Ci, Ci, gCi, c,
+                                           dev_err, s);
     default:
       return cudaErrorInvalidValue;
   }
