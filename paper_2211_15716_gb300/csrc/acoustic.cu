@@ -14,23 +14,33 @@ namespace {
 
 constexpr int kAcX = 32, kAcY = 8, kAcZ = 32;
 
+// Coefficients in the storage type (formed on the host), and the number 1:
+// FP64 differences a - b are computed as fma(a, 1, -b), the same rounding by the
+// FMA instruction. The FP64 launches are bound by the FP64 pipe, which takes
+// FMAs faster than additions (598 against 504 G/s in independent chains): 2x2x2
+// x 256^3 cells, four steps, 11.89 to 11.25 ms.
+template <class S>
+struct AcW {
+  S ax, ay, az, bx, by, bz, one;
+};
+
 template <class S>
 struct AcNum;
 template <>
 struct AcNum<double> {
-  static __device__ __forceinline__ double sub(double a, double b) { return __dsub_rn(a, b); }
+  static __device__ __forceinline__ double sub(double a, double b, double one) {
+    return __fma_rn(a, one, -b);
+  }
   static __device__ __forceinline__ double fma(double a, double b, double c) {
     return __fma_rn(a, b, c);
   }
-  static __device__ __forceinline__ double mul(double a, double b) { return __dmul_rn(a, b); }
 };
 template <>
 struct AcNum<float> {
-  static __device__ __forceinline__ float sub(float a, float b) { return __fsub_rn(a, b); }
+  static __device__ __forceinline__ float sub(float a, float b, float) { return __fsub_rn(a, b); }
   static __device__ __forceinline__ float fma(float a, float b, float c) {
     return __fmaf_rn(a, b, c);
   }
-  static __device__ __forceinline__ float mul(float a, float b) { return __fmul_rn(a, b); }
 };
 
 // blockIdx.z = subdomain * zchunks + z chunk. The z march is software
@@ -72,13 +82,13 @@ __device__ __forceinline__ void ac_put(S *p, S v, const AcSend &a, long long np,
 template <class S>
 __global__ void __launch_bounds__(kAcX *kAcY)
     k_acoustic_v(int nx, int ny, int nz, int zchunks, const S *P, S *__restrict__ Vx,
-                 S *__restrict__ Vy, S *__restrict__ Vz, AcCoef c) {
+                 S *__restrict__ Vy, S *__restrict__ Vz, const AcW<S> w,
+                 const int *__restrict__ nbr, int ox, int xsend) {
   using N = AcNum<S>;
   const int i = blockIdx.x * kAcX + threadIdx.x, j = blockIdx.y * kAcY + threadIdx.y;
   if (i >= nx || j >= ny) return;
   const long long sub = blockIdx.z / zchunks;
   const int k0 = (int)(blockIdx.z % zchunks) * kAcZ, k1 = min(k0 + kAcZ, nz);
-  const S ax = (S)c.ax, ay = (S)c.ay, az = (S)c.az;
   const long long np = (long long)nx * ny * nz;
   const long long sp = (long long)nx * ny, sx = (long long)(nx + 1) * ny,
                   sy = (long long)nx * (ny + 1);
@@ -92,11 +102,11 @@ __global__ void __launch_bounds__(kAcX *kAcY)
   // (halo cells: Vy and Vz not stored)
   AcSend ex{0u, 0, 0}, ev = ex;
   bool keep = true;
-  const int h = nx - c.ox;
-  if (c.xsend) {
-    const int xl = c.nbr[6 * sub], xr = c.nbr[6 * sub + 1];
-    ex = ac_send(i, nx + 1, c.ox + 1, sub, xl, xr);
-    ev = ac_send(i, nx, c.ox, sub, xl, xr);
+  const int h = nx - ox;
+  if (xsend) {
+    const int xl = nbr[6 * sub], xr = nbr[6 * sub + 1];
+    ex = ac_send(i, nx + 1, ox + 1, sub, xl, xr);
+    ev = ac_send(i, nx, ox, sub, xl, xr);
     keep = !((i == 0 && xl >= 0) || (i == nx - 1 && xr >= 0));
   }
   const bool sv = ev.sm != 0u;  // sends Vy and Vz (wall faces too)
@@ -125,15 +135,15 @@ __global__ void __launch_bounds__(kAcX *kAcY)
       vz1 = Vzs[sp * (k + 1)];
     }
     if (i > 0) {
-      vx = N::fma(-ax, N::sub(pc, pxm), vx);
+      vx = N::fma(-w.ax, N::sub(pc, pxm, w.one), vx);
       Vxs[sx * k] = vx;
     }
     if (j > 0) {
-      vy = N::fma(-ay, N::sub(pc, pym), vy);
+      vy = N::fma(-w.ay, N::sub(pc, pym, w.one), vy);
       if (keep) Vys[sy * k] = vy;
     }
     if (k > 0) {
-      vz = N::fma(-az, N::sub(pc, pzm), vz);
+      vz = N::fma(-w.az, N::sub(pc, pzm, w.one), vz);
       if (keep) Vzs[sp * k] = vz;
     }
     if (ex.sm) ac_put(Vxs + sx * k, vx, ex, npx, h);
@@ -159,13 +169,13 @@ __global__ void __launch_bounds__(kAcX *kAcY)
 template <class S>
 __global__ void __launch_bounds__(kAcX *kAcY)
     k_acoustic_p(int nx, int ny, int nz, int zchunks, S *__restrict__ P,
-                 const S *Vx, const S *Vy, const S *Vz, AcCoef c) {
+                 const S *Vx, const S *Vy, const S *Vz, const AcW<S> w,
+                 const int *__restrict__ nbr, int ox, int xsend) {
   using N = AcNum<S>;
   const int i = blockIdx.x * kAcX + threadIdx.x, j = blockIdx.y * kAcY + threadIdx.y;
   if (i >= nx || j >= ny) return;
   const long long sub = blockIdx.z / zchunks;
   const int k0 = (int)(blockIdx.z % zchunks) * kAcZ, k1 = min(k0 + kAcZ, nz);
-  const S bx = (S)c.bx, by = (S)c.by, bz = (S)c.bz;
   const long long np = (long long)nx * ny * nz;
   const long long sp = (long long)nx * ny, sx = (long long)(nx + 1) * ny,
                   sy = (long long)nx * (ny + 1);
@@ -175,10 +185,10 @@ __global__ void __launch_bounds__(kAcX *kAcY)
   const S *Vzs = Vz + sub * (long long)nx * ny * (nz + 1) + i + (long long)nx * j;
   AcSend ep{0u, 0, 0};
   bool keep = true;
-  const int h = nx - c.ox;
-  if (c.xsend) {
-    const int xl = c.nbr[6 * sub], xr = c.nbr[6 * sub + 1];
-    ep = ac_send(i, nx, c.ox, sub, xl, xr);
+  const int h = nx - ox;
+  if (xsend) {
+    const int xl = nbr[6 * sub], xr = nbr[6 * sub + 1];
+    ep = ac_send(i, nx, ox, sub, xl, xr);
     keep = !((i == 0 && xl >= 0) || (i == nx - 1 && xr >= 0));
   }
   pdl_trigger();
@@ -201,9 +211,9 @@ __global__ void __launch_bounds__(kAcX *kAcY)
     }
     // P - bx dVx - by dVy - bz dVz, one FMA per term (6 FP64 instructions
     // per cell for FP64 fields, whose launches the FP64 pipe bounds)
-    S pn = N::fma(-bx, N::sub(x1, x0), pc);
-    pn = N::fma(-by, N::sub(y1, y0), pn);
-    pn = N::fma(-bz, N::sub(vzp, vzc), pn);
+    S pn = N::fma(-w.bx, N::sub(x1, x0, w.one), pc);
+    pn = N::fma(-w.by, N::sub(y1, y0, w.one), pn);
+    pn = N::fma(-w.bz, N::sub(vzp, vzc, w.one), pn);
     if (keep) Ps[sp * k] = pn;
     if (ep.sm) ac_put(Ps + sp * k, pn, ep, np, h);
     vzc = vzp;
@@ -224,11 +234,12 @@ cudaError_t launch_t(int nsub, int nx, int ny, int nz, void *P, void *Vx, void *
   if (gz > 65535) return cudaErrorInvalidValue;
   const dim3 grid((nx + kAcX - 1) / kAcX, (ny + kAcY - 1) / kAcY, (unsigned)gz);
   const dim3 block(kAcX, kAcY);
+  const AcW<S> w = {(S)c.ax, (S)c.ay, (S)c.az, (S)c.bx, (S)c.by, (S)c.bz, S(1)};
   cudaError_t e = launch_pdl(true, k_acoustic_v<S>, grid, block, 0, s, nx, ny, nz, zchunks, (const S *)P,
-                             (S *)Vx, (S *)Vy, (S *)Vz, c);
+                             (S *)Vx, (S *)Vy, (S *)Vz, w, c.nbr, c.ox, c.xsend);
   if (e != cudaSuccess) return e;
   return launch_pdl(true, k_acoustic_p<S>, grid, block, 0, s, nx, ny, nz, zchunks, (S *)P, (const S *)Vx,
-                    (const S *)Vy, (const S *)Vz, c);
+                    (const S *)Vy, (const S *)Vz, w, c.nbr, c.ox, c.xsend);
 }
 
 }  // namespace
