@@ -1,0 +1,33 @@
+// The list of points that the kernels of the emulated FP64 cell leave to the
+// fix-up launch (tma.cu: k_fixup_f64): layout and the entries a warp stages.
+#pragma once
+
+#include <cstddef>
+
+namespace igg {
+namespace {
+
+// A tile set's fix-up buffer (layout in igg_internal.h): the entries, then
+// the entry count and a block counter.
+struct FixEntry {
+  long long p;    // index of the first of 32 consecutive points of a row
+  unsigned bits;  // bit l: point p + l left to the fix-up
+  unsigned pad;
+};
+// Entries a consumer warp stages in shared memory before it reserves their
+// slots in the list with one atomic (a warp waited for each atomic's
+// return, row after row, on fields with many such points).
+constexpr unsigned kFixPend = 16;
+struct FixList {
+  FixEntry *e;
+  unsigned *count, *done;
+  unsigned long long *totals;  // segments and points fixed up since the buffer was made
+};
+__device__ __forceinline__ FixList fix_list(void *fix, size_t cap) {
+  FixEntry *e = reinterpret_cast<FixEntry *>(fix);
+  unsigned *c = reinterpret_cast<unsigned *>(e + cap);
+  return {e, c, c + 1, reinterpret_cast<unsigned long long *>(c + 2)};
+}
+
+}  // namespace
+}  // namespace igg

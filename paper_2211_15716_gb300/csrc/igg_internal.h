@@ -184,7 +184,7 @@ struct TmaTile {
   int zoff;
   int pad[2];
 };
-enum { TMA_WIDE = 0, TMA_WIDE_SWAP = 2 };
+enum { TMA_WIDE = 0, TMA_WIDE_SWAP = 2, TMA_ROWS = 3 };  // (TMA_ROWS: rows.cu)
 // TMA tiles of the box [x0,x1) x rows [r0,r1) x march [m0,m1) (chunks of mb
 // planes) of one array at element offset base whose planes start at plane
 // zoff of the tensor map; tile width Wt, rows Ht, vector width V.
@@ -229,6 +229,19 @@ struct FixBuf {
 };
 size_t tma_fix_cap(const TmaTile *tiles, int ntiles);
 inline size_t tma_fix_bytes(size_t cap) { return cap * 16 + 2 * sizeof(unsigned) + 16; }
+// The fix-up of the launch before it on the stream (c.npts set).
+cudaError_t launch_fixup(FixBuf fix, void *T2, const void *T, const void *Ci, int nx, int ny,
+                         const Coef &c, cudaStream_t s);
+// Row-copy kernel (rows.cu): the full step on grids whose rows are not a
+// multiple of 16 bytes (no tensor map takes their pitch). Tiles as for the TMA
+// kernel with V = 1 (x0 = xb), rows_tile_width points by rows_tile_rows rows.
+constexpr int kRowsMinNx = 32;
+int rows_tile_width(igg_dtype dt);
+int rows_tile_rows(igg_dtype dt);
+cudaError_t rows_prepare(igg_dtype dt, int *ctas_per_sm);
+cudaError_t launch_stencil_rows(igg_dtype dt, const TmaTile *tiles, int ntiles, void *T2,
+                                const void *T, const void *Ci, int nx, int ny, long long nzt,
+                                const Coef &c, unsigned *dev_err, FixBuf fix, cudaStream_t s);
 cudaError_t launch_stencil_tma(igg_dtype dt, int variant, const TmaTile *tiles, int ntiles,
                                void *T2, const void *T, const void *Ci, int nx, int ny,
                                long long nzt, const Coef &c, unsigned *dev_err,
@@ -299,6 +312,7 @@ static inline cudaError_t read_bounds_flag(unsigned *out, bool) {
 #endif
 // the flags of the translation units with checked kernels
 cudaError_t tma_bounds_flag(unsigned *out, bool clear);
+cudaError_t rows_bounds_flag(unsigned *out, bool clear);
 cudaError_t halo_bounds_flag(unsigned *out, bool clear);
 struct HaloJob {
   const PlaneCopy *copies;

@@ -341,13 +341,14 @@ int upload_vec(const std::vector<TT> &v, TileSet *out) {
   return IGG_OK;
 }
 
-int upload_tiles(const TileLists &v, int V, TileSet *out, int tma = -1) {
+// f64: an FP64 set of the TMA or row-copy kernel (it gets a fix-up list)
+int upload_tiles(const TileLists &v, int V, TileSet *out, int tma = -1, bool f64 = false) {
   out->V = V;
   out->tma = tma;
   out->fix = FixBuf();
   if (tma >= 0) {
     if (int rc = upload_vec(v.tma, out)) return rc;
-    if (V == 2 && out->n > 0) {  // FP64: list of the emulated cell's fix-up
+    if (f64 && out->n > 0) {  // FP64: list of the emulated cell's fix-up
       out->fix.cap = tma_fix_cap(v.tma.data(), out->n);
       const size_t bytes = tma_fix_bytes(out->fix.cap);
       cudaError_t e = cudaMalloc(&out->fix.p, bytes);
@@ -379,7 +380,7 @@ struct igg_grid {
   std::vector<int> left, right;  // [nsub*3]
   cudaStream_t hi = nullptr, lo = nullptr, cap = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_hi = nullptr, ev_lo = nullptr, ev_face = nullptr;
-  std::map<int, TileSet> full;                     // keyed by V (1 = scalar tiles)
+  std::map<int, TileSet> full;                     // keyed by full_key
   std::map<int, PartTiles> part;                   // keyed by V (TMA tiles only)
   std::map<std::array<int, 4>, SplitTiles> split;  // keyed by widths and V
   PlaneCopy *copies[3] = {nullptr, nullptr, nullptr};
@@ -460,6 +461,16 @@ int grid_vec(const igg_grid *g, igg_dtype dt) {
 }
 
 // Tiles of one box per subdomain, for the full step.
+// The row-copy kernel takes the full step of the other 3-D grids (rows not a
+// multiple of 16 bytes), down to rows of kRowsMinNx points.
+bool use_rows(const igg_grid *g, int V) {
+  return V == 1 && g->tma_enabled && !low_dim(g) && g->n[0] >= kRowsMinNx;
+}
+
+// Key of the full step's tile tables: the vector width, or, for V = 1, 16 +
+// the dtype (the row-copy kernel's tile width depends on it).
+int full_key(const igg_grid *g, int V, igg_dtype dt) { return use_rows(g, V) ? 16 + (int)dt : V; }
+
 // The full step's TMA tiles of every subdomain. Tile order: for each (z
 // chunk, row block) the tiles of the subdomains that are neighbours in x
 // side by side (measured faster than subdomain after subdomain).
@@ -491,8 +502,9 @@ bool touches_faces(const igg_grid *g, const TmaTile &t) {
          (ex[2] && side(t.m0, t.m1, g->n[2], g->overlap[2]));
 }
 
-int build_full_tiles(igg_grid *g, int V, TileSet **out) {
-  auto it = g->full.find(V);
+int build_full_tiles(igg_grid *g, int V, igg_dtype dt, TileSet **out) {
+  const int key = full_key(g, V, dt);
+  auto it = g->full.find(key);
   if (it != g->full.end()) {
     *out = &it->second;
     return IGG_OK;
@@ -507,8 +519,20 @@ int build_full_tiles(igg_grid *g, int V, TileSet **out) {
   const int zbt = tma ? choose_zb_tma(tma_xy_tiles(1, nx - 1, 1, ny - 1, V, Wt, Ht) * g->nsub,
                                       nz - 2, tma_slots(V))
                       : 0;
+  const bool rows = use_rows(g, V);
   if (tma) {
     full_tma_list(g, V, zbt, Wt, Ht, v.tma);
+  } else if (rows) {
+    const int W = rows_tile_width(dt), H = rows_tile_rows(dt);
+    int per_sm = 1, sms = 152;
+    cudaError_t e = rows_prepare(dt, &per_sm);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, g->device);
+    if (e != cudaSuccess) return cuda_error(e, "row-copy kernel set-up");
+    const long long xyt = (long long)((nx - 2 + W - 1) / W) * ((ny - 2 + H - 1) / H) * g->nsub;
+    const int zbr = choose_zb_tma(xyt, nz - 2, (long long)std::max(1, per_sm) * sms);
+    for (int s = 0; s < g->nsub; ++s)
+      add_box_tma(v.tma, (long long)s * g->nloc, (long long)s * nz, 1, nx - 1, 1, ny - 1, 1, nz - 1,
+                  zbr, 1, W, H);
   } else {
     for (int s = 0; s < g->nsub; ++s)
       add_tiles(v, V, (long long)s * g->nloc, nx, ny, 1, nx - 1, lo_in(ny), hi_in(ny), lo_in(nz),
@@ -516,8 +540,8 @@ int build_full_tiles(igg_grid *g, int V, TileSet **out) {
   }
   zero_absent_strides(g, v.vec);
   TileSet ts;
-  if (int rc = upload_tiles(v, V, &ts, tma ? TMA_WIDE : -1)) return rc;
-  *out = &g->full.emplace(V, ts).first->second;
+  if (int rc = upload_tiles(v, V, &ts, tma ? TMA_WIDE : rows ? TMA_ROWS : -1, dt == IGG_F64)) return rc;
+  *out = &g->full.emplace(key, ts).first->second;
   return IGG_OK;
 }
 
@@ -539,8 +563,8 @@ int build_part_tiles(igg_grid *g, int V, PartTiles **out) {
   TileLists f, in;
   for (const TmaTile &t : all) (touches_faces(g, t) ? f : in).tma.push_back(t);
   PartTiles pt;
-  if (int rc = upload_tiles(f, V, &pt.face, TMA_WIDE)) return rc;
-  if (int rc = upload_tiles(in, V, &pt.inner, TMA_WIDE)) {
+  if (int rc = upload_tiles(f, V, &pt.face, TMA_WIDE, V == 2)) return rc;
+  if (int rc = upload_tiles(in, V, &pt.inner, TMA_WIDE, V == 2)) {
     free_tiles(pt.face);
     return rc;
   }
@@ -619,10 +643,10 @@ int build_split_tiles(igg_grid *g, const int w[3], int V, SplitTiles **out) {
         break;
       }
       TileSet ts;
-      if ((rc = upload_tiles(*pt.first, V, &ts, pt.second)) != IGG_OK) break;
+      if ((rc = upload_tiles(*pt.first, V, &ts, pt.second, V == 2)) != IGG_OK) break;
       st.boundary.push_back(ts);
     }
-    if (rc == IGG_OK) rc = upload_tiles(vi, V, &st.inner, TMA_WIDE);
+    if (rc == IGG_OK) rc = upload_tiles(vi, V, &st.inner, TMA_WIDE, V == 2);
   } else {
     for (int s = 0; s < g->nsub; ++s) {
       const long long base = (long long)s * g->nloc;
@@ -653,6 +677,9 @@ int build_split_tiles(igg_grid *g, const int w[3], int V, SplitTiles **out) {
 
 cudaError_t launch_tiles(const igg_grid *g, int V, igg_dtype dt, const TileSet &ts, void *T2,
                          const void *T, const void *Ci, const Coef &c, cudaStream_t s) {
+  if (ts.tma == TMA_ROWS)
+    return launch_stencil_rows(dt, (const TmaTile *)ts.dev, ts.n, T2, T, Ci, g->n[0], g->n[1],
+                               (long long)g->nsub * g->n[2], c, g->dev_err, ts.fix, s);
   if (ts.tma >= 0)
     return launch_stencil_tma(dt, ts.tma, (const TmaTile *)ts.dev, ts.n, T2, T, Ci, g->n[0],
                               g->n[1], (long long)g->nsub * g->n[2], c, g->dev_err, ts.fix, s);
@@ -896,7 +923,7 @@ int enqueue_step(igg_grid *g, const int *widths, void *T2, const void *T, const 
   }
   if (!widths) {
     TileSet *full = nullptr;
-    if (int rc = build_full_tiles(g, V, &full)) return rc;
+    if (int rc = build_full_tiles(g, V, dt, &full)) return rc;
     c.ends = with_halo && any_halo(g) ? 1 : 0;
     {
       NvtxRange r("stencil");
@@ -1360,7 +1387,7 @@ int igg_run(igg_grid *g, int nt, const int widths[3], void *T, void *T2, const v
       if (int rc = build_part_tiles(g, V, &pt)) return rc;
     } else {
       TileSet *full = nullptr;
-      if (int rc = build_full_tiles(g, V, &full)) return rc;
+      if (int rc = build_full_tiles(g, V, dt, &full)) return rc;
     }
     const GraphKey key(T, T2, Ci, (int)dt, widths ? 1 : 0, widths ? widths[0] : 0,
                        widths ? widths[1] : 0, widths ? widths[2] : 0, c.wx, c.wy, c.wz, c.wc);
@@ -1727,6 +1754,9 @@ int igg_bounds_status(unsigned *status, int clear) {
   unsigned a = 0u, b = 0u;
   cudaError_t e = tma_bounds_flag(&a, clear != 0);
   if (e == cudaSuccess) e = halo_bounds_flag(&b, clear != 0);
+  unsigned r = 0u;
+  if (e == cudaSuccess) e = rows_bounds_flag(&r, clear != 0);
+  b |= r;
   if (e != cudaSuccess) return cuda_error(e, "bounds status");
   *status = (a | b) ? IGG_DEV_ERR_BOUNDS : 0u;
   return IGG_OK;

@@ -27,6 +27,7 @@
 #include <mutex>
 
 #include "cell.cuh"
+#include "fixlist.cuh"
 #include "igg_internal.h"
 #include "tma_util.cuh"
 
@@ -72,27 +73,6 @@ struct TmaShape {
 template <class S>
 __device__ __forceinline__ void lds_vec(const S *p, Vec<S> &o) {
   unpack(*reinterpret_cast<const uint4 *>(p), o);
-}
-// A tile set's fix-up buffer (layout in igg_internal.h): the entries, then
-// the entry count and a block counter.
-struct FixEntry {
-  long long p;    // index of the first of 32 consecutive points of a row
-  unsigned bits;  // bit l: point p + l left to the fix-up
-  unsigned pad;
-};
-// Entries a consumer warp stages in shared memory before it reserves their
-// slots in the list with one atomic (a warp waited for each atomic's
-// return, row after row, on fields with many such points).
-constexpr unsigned kFixPend = 16;
-struct FixList {
-  FixEntry *e;
-  unsigned *count, *done;
-  unsigned long long *totals;  // segments and points fixed up since the buffer was made
-};
-__device__ __forceinline__ FixList fix_list(void *fix, size_t cap) {
-  FixEntry *e = reinterpret_cast<FixEntry *>(fix);
-  unsigned *c = reinterpret_cast<unsigned *>(e + cap);
-  return {e, c, c + 1, reinterpret_cast<unsigned long long *>(c + 2)};
 }
 constexpr int kFixupBlocks = 8 * 152;
 
@@ -631,6 +611,13 @@ __global__ void __launch_bounds__(256)
   }
 }
 
+template <int NG>
+cudaError_t launch_fixup_t(FixBuf fix, void *T2, const void *T, const void *Ci, int nx, int ny,
+                           const Coef &c, cudaStream_t s) {
+  return launch_pdl(pdl_on(c.npts), k_fixup_f64<NG>, kFixupBlocks, 256, 0, s, fix.p, fix.cap,
+                    (double *)T2, (const double *)T, (const double *)Ci, nx, ny, c);
+}
+
 template <class S, class Shp, bool SWAP, int MODE>
 cudaError_t prepare_t(int *ctas_per_sm) {
   using Sh = TmaShape<S, Shp::LPR, Shp::H>;
@@ -659,8 +646,7 @@ cudaError_t launch_t(const TmaTile *tiles, int ntiles, void *T2, const void *T, 
                              32 * (Sh::CONSUMERS + 1), Sh::SMEM, s, mT, mC, tiles, (S *)T2, nx, ny,
                              cc, dev_err, fix.p, fix.cap, TmaBatch());
   if (e == cudaSuccess && is_emu(MODE))
-    e = launch_pdl(pdl_on(cc.npts), k_fixup_f64<emu_groups(MODE)>, kFixupBlocks, 256, 0, s, fix.p, fix.cap, (double *)T2,
-                   (const double *)T, (const double *)Ci, nx, ny, cc);
+    e = launch_fixup_t<emu_groups(MODE)>(fix, T2, T, Ci, nx, ny, cc, s);
   return e;
 }
 
@@ -836,6 +822,15 @@ cudaError_t launch_stencil_tma_batch(igg_dtype dt, const TmaTile *tiles, int nti
   return cudaErrorInvalidValue;
 }
 
+
+cudaError_t launch_fixup(FixBuf fix, void *T2, const void *T, const void *Ci, int nx, int ny,
+                         const Coef &c, cudaStream_t s) {
+  switch (weight_groups(c.wx, c.wy, c.wz)) {
+    case 1: return launch_fixup_t<1>(fix, T2, T, Ci, nx, ny, c, s);
+    case 2: return launch_fixup_t<2>(fix, T2, T, Ci, nx, ny, c, s);
+    default: return launch_fixup_t<3>(fix, T2, T, Ci, nx, ny, c, s);
+  }
+}
 
 size_t tma_fix_cap(const TmaTile *tiles, int ntiles) {
   size_t cap = 0;
