@@ -242,10 +242,12 @@ cudaError_t rows_prepare(igg_dtype dt, int *ctas_per_sm);
 cudaError_t launch_stencil_rows(igg_dtype dt, const TmaTile *tiles, int ntiles, void *T2,
                                 const void *T, const void *Ci, int nx, int ny, long long nzt,
                                 const Coef &c, unsigned *dev_err, FixBuf fix, cudaStream_t s);
+// inl: FP64 fields with the emulated cell fix up their points in the stencil
+// launch itself (small grids; TMA_WIDE)
 cudaError_t launch_stencil_tma(igg_dtype dt, int variant, const TmaTile *tiles, int ntiles,
                                void *T2, const void *T, const void *Ci, int nx, int ny,
                                long long nzt, const Coef &c, unsigned *dev_err,
-                               FixBuf fix, cudaStream_t s);
+                               FixBuf fix, bool inl, cudaStream_t s);
 
 // Staggered-grid acoustics (acoustic.cu): coefficients dt/(rho dd) of the
 // velocity update and dt K/dd of the pressure update, formed on the host in

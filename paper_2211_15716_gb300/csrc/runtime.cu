@@ -93,6 +93,7 @@ struct TileSet {
   int n = 0;
   int V = 1;
   int tma = -1;
+  bool inl = false;  // small grid: no fix-up launch (FP64 TMA tile sets)
   FixBuf fix;  // fix-up list (FP64 TMA tile sets)
 };
 
@@ -516,9 +517,15 @@ int build_full_tiles(igg_grid *g, int V, igg_dtype dt, TileSet **out) {
   const bool tma = use_tma(g, V);
   const int Wt = tma ? tma_tile_width(dtype_of_vec(V), TMA_WIDE) : 0;
   const int Ht = tma ? tma_tile_rows(dtype_of_vec(V), TMA_WIDE) : 0;
-  const int zbt = tma ? choose_zb_tma(tma_xy_tiles(1, nx - 1, 1, ny - 1, V, Wt, Ht) * g->nsub,
-                                      nz - 2, tma_slots(V))
-                      : 0;
+  const long long xyt = tma ? tma_xy_tiles(1, nx - 1, 1, ny - 1, V, Wt, Ht) * g->nsub : 0;
+  int zbt = tma ? choose_zb_tma(xyt, nz - 2, tma_slots(V)) : 0;
+  // FP64 grids that make one wave of two CTAs per SM with tiles of up to
+  // kInlPlanes planes fix up in the stencil launch: the planes a tile fixes up
+  // cost it about a microsecond each, a fix-up launch of its own four or five
+  constexpr int kInlPlanes = 4;
+  const long long wave2 = 2 * (tma_slots(V) / 3);
+  const bool inl = tma && V == 2 && xyt * ((nz - 2 + kInlPlanes - 1) / kInlPlanes) <= wave2;
+  if (inl) zbt = choose_zb_tma(xyt, nz - 2, wave2);
   const bool rows = use_rows(g, V);
   if (tma) {
     full_tma_list(g, V, zbt, Wt, Ht, v.tma);
@@ -541,6 +548,7 @@ int build_full_tiles(igg_grid *g, int V, igg_dtype dt, TileSet **out) {
   zero_absent_strides(g, v.vec);
   TileSet ts;
   if (int rc = upload_tiles(v, V, &ts, tma ? TMA_WIDE : rows ? TMA_ROWS : -1, dt == IGG_F64)) return rc;
+  ts.inl = inl;
   *out = &g->full.emplace(key, ts).first->second;
   return IGG_OK;
 }
@@ -682,7 +690,7 @@ cudaError_t launch_tiles(const igg_grid *g, int V, igg_dtype dt, const TileSet &
                                (long long)g->nsub * g->n[2], c, g->dev_err, ts.fix, s);
   if (ts.tma >= 0)
     return launch_stencil_tma(dt, ts.tma, (const TmaTile *)ts.dev, ts.n, T2, T, Ci, g->n[0],
-                              g->n[1], (long long)g->nsub * g->n[2], c, g->dev_err, ts.fix, s);
+                              g->n[1], (long long)g->nsub * g->n[2], c, g->dev_err, ts.fix, ts.inl, s);
   if (V > 1) return launch_stencil_vec(dt, (const VTile *)ts.dev, ts.n, T2, T, Ci, c, nullptr, s);
   return launch_stencil(dt, (const Tile *)ts.dev, ts.n, T2, T, Ci, c, nullptr, s);
 }

@@ -199,6 +199,76 @@ __device__ __forceinline__ void compute_vec<double, MODE_EMU + 2>(
   compute_vec_emu<1>(c, left, right, ym, yp, zm, zp, ci, w, out, ok);
 }
 
+// ---------------------------------------------------------------------------
+// Small grids (INL): the points that the fast path of one warp's two rows of a
+// plane did not take, fixed up by the warp itself from the planes in shared
+// memory, over what the rows' vector stores left there (the same choice and
+// arithmetic as the fix-up launch). The refused points are dealt out to the
+// lanes (their indices compacted through shared memory), 32 at a time.
+//
+// The steps of a small grid are bound by the latency of their launches, so one
+// launch instead of two is what counts (one 64^3 array, 100 steps: 1.17 to 0.51 ms).
+// On larger grids the fix-up stays a launch of its own: a plane that a warp
+// fixes up takes it about a microsecond longer, which the tiles along a shell
+// add up over their planes (misfit gradient at 256^3, 48 steps: 23.5 against
+// 21.6 ms), and in the march of three CTAs per SM there are no registers for it
+// (10.97 against 10.72 ms for ten steps of 2x2x2 x 512x256x256).
+// ---------------------------------------------------------------------------
+struct FixShared {
+  unsigned segs, pts;           // row segments and points fixed up by this CTA
+  unsigned char list[8][128];   // per consumer warp: refused points (64 row + x)
+};
+
+static_assert(sizeof(FixShared) <= 8 * kFixPend * sizeof(FixEntry), "in the staging's place");
+
+// Tm, Tc, Tn, Cn: the T planes m - 1, m, m + 1 and the Ci plane; warp: the
+// consumer warp, whose rows are warp and warp + H / 2; d0: the first row's place
+// in T2, the second row dj elements further. def: bits 0, 1 the first row's two
+// points of this lane, bits 2, 3 the second's.
+template <int NG, bool SWAP>
+__device__ __forceinline__ void emu_fix_rows(const double *Tm, const double *Tc, const double *Tn,
+                                             const double *Cn, int warp, double *d0, long long dj,
+                                             unsigned def, const W<double> &w, FixShared *fs) {
+  using Sh = TmaShape<double, 32, 16>;
+  constexpr unsigned kAll = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  const unsigned lt = (1u << lane) - 1u;
+  unsigned char *list = fs->list[warp];
+  int total = 0;
+  unsigned segs = 0u;
+#pragma unroll
+  for (int j = 0; j < 2; ++j) {
+    const unsigned b0 = __ballot_sync(kAll, def >> (2 * j) & 1u);
+    const unsigned b1 = __ballot_sync(kAll, def >> (2 * j) & 2u), b = b0 | b1;
+    if (def >> (2 * j) & 1u) list[total + __popc(b0 & lt)] = (unsigned char)(64 * j + 2 * lane);
+    total += __popc(b0);
+    if (def >> (2 * j) & 2u) list[total + __popc(b1 & lt)] = (unsigned char)(64 * j + 2 * lane + 1);
+    total += __popc(b1);
+    segs += ((b & 0xffffu) ? 1u : 0u) + ((b >> 16) ? 1u : 0u);  // 32-point segments
+  }
+  if (lane == 0) {
+    atomicAdd(&fs->pts, (unsigned)total);
+    atomicAdd(&fs->segs, segs);
+  }
+  __syncwarp();  // the list, and the rows' vector stores before the stores below
+  for (int i = lane; i < total; i += 32) {
+    const int q = list[i], j = q >> 6, x = q & 63, r = warp + j * (Sh::H / 2);
+    const int o = (r + 1) * Sh::BW + Sh::V + x;
+    const double *pc = Tc + o;
+    const double up = pc[-Sh::BW], dn = pc[Sh::BW], m = Tm[o], n = Tn[o], ci = Cn[r * Sh::W + x];
+    const double tn[6] = {pc[-1],        pc[1],         SWAP ? m : up,
+                          SWAP ? n : dn, SWAP ? up : m, SWAP ? dn : n};
+    unsigned long long nb[6];
+#pragma unroll
+    for (int k = 0; k < 6; ++k) nb[k] = dbits(tn[k]);
+    bool ok;
+    double v = cell_emu_aligned<NG>(*pc, nb, ci, w, ok);
+    if (!ok) v = cell_f64(*pc, tn[0], tn[1], tn[2], tn[3], tn[4], tn[5], ci, w);
+    d0[(j ? dj : 0) + x] = v;
+  }
+  __syncwarp();  // the list before its next use
+}
+
 // SWAP = false: rows along y, march along z (box {BW, BH, 1}); SWAP = true:
 // rows along z, march along y (box {BW, 1, BH}), for boxes thin in y. The
 // cell arithmetic gets the y and z neighbour pairs in their own slots either
@@ -207,8 +277,11 @@ __device__ __forceinline__ void compute_vec<double, MODE_EMU + 2>(
 // BATCH: independent problems of the batched form; a tile's problem (pad[0])
 // gives its tensor maps, row pitch, ny and coefficients (TmaBatch) in place
 // of mapT, mapC, nx, ny and c0.
-template <class S, int LPR_, int H_, bool SWAP, int MODE, bool BATCH = false>
-__global__ void __launch_bounds__(32 * 9, IGG_TMA_MIN_BLOCKS)
+//
+// INL (emulated cell): the warps fix up their rows themselves (emu_fix_rows), a
+// stage is freed a step later (its T plane is m - 1 then), two CTAs per SM.
+template <class S, int LPR_, int H_, bool SWAP, int MODE, bool BATCH = false, bool INL = false>
+__global__ void __launch_bounds__(32 * 9, INL ? 2 : IGG_TMA_MIN_BLOCKS)
     k_stencil_tma(const __grid_constant__ CUtensorMap mapT, const __grid_constant__ CUtensorMap mapC,
                   const TmaTile *__restrict__ tiles, S *__restrict__ T2, int nx, int ny, Coef c0,
                   unsigned *__restrict__ dev_err, void *__restrict__ fix, size_t fix_cap,
@@ -223,6 +296,7 @@ __global__ void __launch_bounds__(32 * 9, IGG_TMA_MIN_BLOCKS)
   volatile int *flags = reinterpret_cast<volatile int *>(smem + NS * Sh::STAGE + 2 * NS * 8);
   // flags[0]: abort; flags[1]: loads issued; flags[2]: loads consumed
 
+  FixShared *fs = reinterpret_cast<FixShared *>(smem + Sh::PEND);  // (INL)
   const TmaTile t = tiles[blockIdx.x];
   const int K = (t.m1 - t.m0) + 2;
   const CUtensorMap *pmT = &mapT, *pmC = &mapC;
@@ -243,6 +317,7 @@ __global__ void __launch_bounds__(32 * 9, IGG_TMA_MIN_BLOCKS)
     flags[0] = 0;
     flags[1] = 0;
     flags[2] = 0;
+    if constexpr (INL) fs->segs = fs->pts = 0u;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
@@ -322,7 +397,7 @@ __global__ void __launch_bounds__(32 * 9, IGG_TMA_MIN_BLOCKS)
 #pragma unroll
       for (int j = 0; j < Sh::RPT; ++j) lds_vec(Tb + (rowi[j] + 1) * Sh::BW + V + sl * V, zm[j]);
       __syncwarp();
-      if (lane == 0) mbar_arrive(empty0);
+      if (!INL && lane == 0) mbar_arrive(empty0);
     }
     int consumed = 2;
     // the warp's staged fix-up entries (emulated FP64 cell)
@@ -357,6 +432,7 @@ __global__ void __launch_bounds__(32 * 9, IGG_TMA_MIN_BLOCKS)
       const S *Tc = reinterpret_cast<const S *>(smem + s * Sh::STAGE);
       const S *Tn = reinterpret_cast<const S *>(smem + s1 * Sh::STAGE);
       const S *Cn = reinterpret_cast<const S *>(smem + s1 * Sh::STAGE + Sh::TBA);
+      unsigned def = 0u;  // (INL) points left to emu_fix_rows
 #pragma unroll
       for (int j = 0; j < Sh::RPT; ++j) {
         const int r = rowi[j];
@@ -407,7 +483,10 @@ __global__ void __launch_bounds__(32 * 9, IGG_TMA_MIN_BLOCKS)
               if (inm >> i & 1u) Num<S>::st(dst + i, out.v[i]);
           }
         }
-        if constexpr (is_emu(MODE)) {
+        if constexpr (INL) {
+          static_assert(is_emu(MODE) && LPR == 32 && V == 2 && Sh::RPT == 2, "two rows per warp");
+          if (comp[j]) def |= (~okm & inm) << (2 * j);
+        } else if constexpr (is_emu(MODE)) {
           // The warp owns the whole row (one row per warp, two points per
           // lane): it lists each 32-point segment of the row with points
           // the fast path did not take (its first point and a bit mask).
@@ -435,13 +514,27 @@ __global__ void __launch_bounds__(32 * 9, IGG_TMA_MIN_BLOCKS)
         }
         zm[j] = c;
       }
+      if constexpr (INL) {
+        if (__any_sync(0xffffffffu, def != 0u))
+          emu_fix_rows<emu_groups(MODE), SWAP>(
+              reinterpret_cast<const S *>(smem + (k - 1) % NS * Sh::STAGE), Tc, Tn, Cn, warp,
+              T2 + t.base + t.x0 + srow * (t.r0 + warp) + smarch * m, srow * (Sh::H / 2), def, w, fs);
+      }
       __syncwarp();
-      if (lane == 0) mbar_arrive(empty0 + 8 * s);
+      // load k's stage (INL: load k - 1's) back to the producer
+      if (lane == 0) mbar_arrive(empty0 + 8 * (INL ? (k - 1) % NS : s));
     }
-    if constexpr (is_emu(MODE)) flush();
+    if constexpr (is_emu(MODE) && !INL) flush();
     if (warp == 0 && lane == 0) flags[2] = consumed;
   }
   __syncthreads();
+  if constexpr (INL) {
+    if (threadIdx.x == 0 && fs->pts) {
+      const FixList fl = fix_list(fix, fix_cap);
+      atomicAdd(fl.totals, (unsigned long long)fs->segs);
+      atomicAdd(fl.totals + 1, (unsigned long long)fs->pts);
+    }
+  }
   // After an abort, wait (bounded) for copies issued but never consumed, so
   // that no bulk copy writes into this CTA's shared memory after it exits.
   if (threadIdx.x == 0 && flags[0]) {
@@ -626,13 +719,18 @@ cudaError_t prepare_t(int *ctas_per_sm) {
   if (e == cudaSuccess && ctas_per_sm)
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas_per_sm, kern, 32 * (Sh::CONSUMERS + 1),
                                                       Sh::SMEM);
+  if constexpr (is_emu(MODE) && !SWAP) {
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(k_stencil_tma<S, Shp::LPR, Shp::H, SWAP, MODE, false, true>,
+                               cudaFuncAttributeMaxDynamicSharedMemorySize, Sh::SMEM);
+  }
   return e;
 }
 
 template <class S, class Shp, bool SWAP, int MODE>
 cudaError_t launch_t(const TmaTile *tiles, int ntiles, void *T2, const void *T, const void *Ci,
                      int nx, int ny, long long nzt, const Coef &c, unsigned *dev_err,
-                     FixBuf fix, cudaStream_t s) {
+                     FixBuf fix, bool inl, cudaStream_t s) {
   using Sh = TmaShape<S, Shp::LPR, Shp::H>;
   CUtensorMap mT, mC;
   const bool ok = SWAP ? encode<S>(&mT, T, nx, ny, nzt, Sh::BW, 1, Sh::BH) &&
@@ -642,6 +740,12 @@ cudaError_t launch_t(const TmaTile *tiles, int ntiles, void *T2, const void *T, 
   if (!ok) return cudaErrorInvalidValue;
   Coef cc = c;
   cc.npts = (long long)nx * ny * nzt;
+  if constexpr (is_emu(MODE) && !SWAP) {
+    if (inl)
+      return launch_pdl(true, k_stencil_tma<S, Shp::LPR, Shp::H, SWAP, MODE, false, true>, ntiles,
+                        32 * (Sh::CONSUMERS + 1), Sh::SMEM, s, mT, mC, tiles, (S *)T2, nx, ny, cc,
+                        dev_err, fix.p, fix.cap, TmaBatch());
+  }
   cudaError_t e = launch_pdl(pdl_on(cc.npts), k_stencil_tma<S, Shp::LPR, Shp::H, SWAP, MODE>, ntiles,
                              32 * (Sh::CONSUMERS + 1), Sh::SMEM, s, mT, mC, tiles, (S *)T2, nx, ny,
                              cc, dev_err, fix.p, fix.cap, TmaBatch());
@@ -676,39 +780,39 @@ cudaError_t prepare_v(int variant, int *ctas) {
 template <class S, bool SWAP>
 cudaError_t launch_m(const TmaTile *tiles, int ntiles, void *T2, const void *T, const void *Ci,
                      int nx, int ny, long long nzt, const Coef &c, unsigned *dev_err,
-                     FixBuf fix, cudaStream_t s) {
+                     FixBuf fix, bool inl, cudaStream_t s) {
   if constexpr (sizeof(S) == 8) {
     if (c.f64_emu) {
       if (!fix.p) return cudaErrorInvalidValue;
       switch (weight_groups(c.wx, c.wy, c.wz)) {
         case 1:
           return launch_t<S, WideShape<S>, SWAP, emu_mode(1)>(tiles, ntiles, T2, T, Ci, nx, ny,
-                                                              nzt, c, dev_err, fix, s);
+                                                              nzt, c, dev_err, fix, inl, s);
         case 2:
           return launch_t<S, WideShape<S>, SWAP, emu_mode(2)>(tiles, ntiles, T2, T, Ci, nx, ny,
-                                                              nzt, c, dev_err, fix, s);
+                                                              nzt, c, dev_err, fix, inl, s);
         default:
           return launch_t<S, WideShape<S>, SWAP, emu_mode(3)>(tiles, ntiles, T2, T, Ci, nx, ny,
-                                                              nzt, c, dev_err, fix, s);
+                                                              nzt, c, dev_err, fix, inl, s);
       }
     }
     return launch_t<S, WideShape<S>, SWAP, MODE_F64>(tiles, ntiles, T2, T, Ci, nx, ny, nzt, c,
-                                                     dev_err, fix, s);
+                                                     dev_err, fix, inl, s);
   } else {
     return launch_t<S, WideShape<S>, SWAP, MODE_CELL>(tiles, ntiles, T2, T, Ci, nx, ny, nzt, c,
-                                                      dev_err, fix, s);
+                                                      dev_err, fix, inl, s);
   }
 }
 
 template <class S>
 cudaError_t launch_v(int variant, const TmaTile *tiles, int ntiles, void *T2, const void *T,
                      const void *Ci, int nx, int ny, long long nzt, const Coef &c,
-                     unsigned *dev_err, FixBuf fix, cudaStream_t s) {
+                     unsigned *dev_err, FixBuf fix, bool inl, cudaStream_t s) {
   switch (variant) {
     case TMA_WIDE:
-      return launch_m<S, false>(tiles, ntiles, T2, T, Ci, nx, ny, nzt, c, dev_err, fix, s);
+      return launch_m<S, false>(tiles, ntiles, T2, T, Ci, nx, ny, nzt, c, dev_err, fix, inl, s);
     case TMA_WIDE_SWAP:
-      return launch_m<S, true>(tiles, ntiles, T2, T, Ci, nx, ny, nzt, c, dev_err, fix, s);
+      return launch_m<S, true>(tiles, ntiles, T2, T, Ci, nx, ny, nzt, c, dev_err, fix, inl, s);
   }
   return cudaErrorInvalidValue;
 }
@@ -854,18 +958,18 @@ cudaError_t tma_prepare(igg_dtype dt, int variant, int *ctas_per_sm) {
 cudaError_t launch_stencil_tma(igg_dtype dt, int variant, const TmaTile *tiles, int ntiles,
                                void *T2, const void *T, const void *Ci, int nx, int ny,
                                long long nzt, const Coef &c, unsigned *dev_err,
-                               FixBuf fix, cudaStream_t s) {
+                               FixBuf fix, bool inl, cudaStream_t s) {
   if (ntiles <= 0) return cudaSuccess;
   switch (dt) {
     case IGG_F64:
-      return launch_v<double>(variant, tiles, ntiles, T2, T, Ci, nx, ny, nzt, c, dev_err, fix,
+      return launch_v<double>(variant, tiles, ntiles, T2, T, Ci, nx, ny, nzt, c, dev_err, fix, inl,
                               s);
     case IGG_F32:
-      return launch_v<float>(variant, tiles, ntiles, T2, T, Ci, nx, ny, nzt, c, dev_err, fix,
+      return launch_v<float>(variant, tiles, ntiles, T2, T, Ci, nx, ny, nzt, c, dev_err, fix, inl,
                              s);
     case IGG_BF16:
       return launch_v<__nv_bfloat16>(variant, tiles, ntiles, T2, T, Ci, nx, ny, nzt, c, dev_err,
-                                     fix, s);
+                                     fix, inl, s);
   }
   return cudaErrorInvalidValue;
 }
