@@ -232,16 +232,16 @@ inline size_t tma_fix_bytes(size_t cap) { return cap * 16 + 2 * sizeof(unsigned)
 // The fix-up of the launch before it on the stream (c.npts set).
 cudaError_t launch_fixup(FixBuf fix, void *T2, const void *T, const void *Ci, int nx, int ny,
                          const Coef &c, cudaStream_t s);
-// Row-copy kernel (rows.cu): the full step on grids whose rows are not a
-// multiple of 16 bytes (no tensor map takes their pitch). Tiles as for the TMA
+// Row-copy kernel (rows.cu): the full FP64 step on grids of odd row length (no
+// tensor map takes their pitch). Tiles as for the TMA
 // kernel with V = 1 (x0 = xb), rows_tile_width points by rows_tile_rows rows.
 constexpr int kRowsMinNx = 32;
-int rows_tile_width(igg_dtype dt);
-int rows_tile_rows(igg_dtype dt);
-cudaError_t rows_prepare(igg_dtype dt, int *ctas_per_sm);
-cudaError_t launch_stencil_rows(igg_dtype dt, const TmaTile *tiles, int ntiles, void *T2,
-                                const void *T, const void *Ci, int nx, int ny, long long nzt,
-                                const Coef &c, unsigned *dev_err, FixBuf fix, cudaStream_t s);
+int rows_tile_width();
+int rows_tile_rows();
+cudaError_t rows_prepare(int *ctas_per_sm);
+cudaError_t launch_stencil_rows(const TmaTile *tiles, int ntiles, void *T2, const void *T,
+                                const void *Ci, int nx, int ny, long long nzt, const Coef &c,
+                                unsigned *dev_err, FixBuf fix, cudaStream_t s);
 // inl: FP64 fields with the emulated cell fix up their points in the stencil
 // launch itself (small grids; TMA_WIDE)
 cudaError_t launch_stencil_tma(igg_dtype dt, int variant, const TmaTile *tiles, int ntiles,

@@ -1,6 +1,7 @@
-// Row-copy stencil kernel: the full step on 3-D grids whose rows are not a
-// multiple of 16 bytes (255 or 127 points, say), which no tensor map takes (a
-// pitch is a multiple of 16 bytes) and whose rows start at any alignment.
+// Row-copy stencil kernel: the full FP64 step on 3-D grids of odd row length
+// (255 or 127 points, say), whose rows are not a multiple of 16 bytes: no tensor
+// map takes them (a pitch is a multiple of 16 bytes), and they start at either
+// alignment.
 //
 // What bounds it: with plain loads, one point per thread and step in flight, it
 // was the latency of the loads (2x2x2 x 255x127x129 FP64, ten steps: 2.57 ms,
@@ -8,13 +9,16 @@
 // keeps several planes of a tile in flight with bulk copies, here one untiled
 // cp.async.bulk per row, issued by a lane each: the row from the 16-byte
 // boundary at or before its first point, so that it lies in its shared-memory
-// row with a shift of 0 .. V - 1 points (V = 16 bytes in points), the same for
+// row with a shift of 0 or 1 points (V = 2 points are 16 bytes), the same for
 // producer and consumers, who both get it from the row's index. A lane of a
 // consumer warp takes the points lane, lane + 32, .. of its row: shared-memory
 // loads and global stores of one point each stay contiguous over the warp at
 // any shift. The producer's copies of a row each bound it then (the consumers
 // wait for them): FP64 tiles of 64 points by 16 rows (512 bytes a copy) took 2.21 ms,
-// of 128 by 8 2.08 with two CTAs per SM and 1.81 with three.
+// of 128 by 8 2.08 with two CTAs per SM and 1.81 with three. The same on FP32 and
+// BF16 fields, whose copies of a row are a half and a quarter as long, took
+// 1.11 and 1.14 ms where the scalar kernel takes 0.93 and 0.79: theirs stay
+// with the scalar kernel.
 //
 // Ring protocol as in the TMA kernel: load k brings T plane m0 - 1 + k and Ci
 // plane m0 - 2 + k into stage k % NS (full[s]: count 1 + transaction bytes;
@@ -39,24 +43,23 @@ namespace {
 // eight)
 constexpr unsigned kRowsPend = 8;
 
-template <class S>
-struct RowsShape {
-  static constexpr int V = 16 / (int)sizeof(S);
+struct Sh {
+  static constexpr int V = 2;                           // points per 16 bytes
   static constexpr int P = 4;                           // points per lane and row
   static constexpr int W = 32 * P;                      // points per row of a tile
   static constexpr int BW = (W + 2 + V - 1 + V - 1) / V * V;  // T row in shared memory
   static constexpr int CW = (W + V - 1 + V - 1) / V * V;      // Ci row
-  static constexpr int H = sizeof(S) == 8 ? 8 : 16;     // rows of a tile
+  static constexpr int H = 8;                            // rows of a tile
   static constexpr int BH = H + 2;
   static constexpr int NS = 4;
   static constexpr int CONSUMERS = 8;
   static constexpr int RPT = H / CONSUMERS;             // rows per consumer warp
-  static constexpr int TB = BW * BH * (int)sizeof(S);   // (multiples of 16 bytes)
-  static constexpr int CB = CW * H * (int)sizeof(S);
+  static constexpr int TB = BW * BH * 8;                  // (multiples of 16 bytes)
+  static constexpr int CB = CW * H * 8;
   static constexpr int STAGE = TB + CB;
   static constexpr int BARS = NS * STAGE;
   static constexpr int PEND = BARS + 2 * NS * 8 + 64;
-  static constexpr int SMEM = PEND + (sizeof(S) == 8 ? CONSUMERS * (int)kRowsPend * 16 : 0);
+  static constexpr int SMEM = PEND + CONSUMERS * (int)kRowsPend * 16;
   static_assert(H % CONSUMERS == 0 && V < kRowsMinNx, "tile");
   static_assert(3 * (SMEM + 1024) <= 228 * 1024, "three CTAs per SM");
   static_assert(BH <= 32 && H <= 32, "one copy per lane");
@@ -71,14 +74,13 @@ __device__ __forceinline__ void bulk_row(unsigned dst, const void *src, unsigned
       : "memory");
 }
 
-// MODE 0: cell() (FP32, BF16); FP64: 1 the FP64 cell, 2 + (3 - NG) the
-// emulated cell's fast path with NG weight groups
-template <class S, int MODE>
+// MODE 1: the FP64 cell; 2 + (3 - NG): the emulated cell's fast path with NG
+// weight groups
+template <int MODE>
 __global__ void __launch_bounds__(32 * 9, 3)
-    k_stencil_rows(const TmaTile *__restrict__ tiles, S *T2, const S *T, const S *Ci, int nx, int ny,
+    k_stencil_rows(const TmaTile *__restrict__ tiles, double *T2, const double *T,
+                   const double *Ci, int nx, int ny,
                    Coef c0, unsigned *dev_err, void *fix, size_t fix_cap) {
-  using Sh = RowsShape<S>;
-  using C = typename Num<S>::C;
   constexpr int V = Sh::V, NS = Sh::NS, P = Sh::P;
   constexpr bool EMU = MODE >= 2;
   extern __shared__ __align__(128) unsigned char smem[];
@@ -137,20 +139,20 @@ __global__ void __launch_bounds__(32 * 9, 3)
       }
       bT = min(bT, lim);
       bC = min(bC, lim);
-      const unsigned nT = hasT && bT > aT ? (unsigned)(bT - aT) * (unsigned)sizeof(S) : 0u;
-      const unsigned nC = k >= 2 && hasC && bC > aC ? (unsigned)(bC - aC) * (unsigned)sizeof(S) : 0u;
+      const unsigned nT = hasT && bT > aT ? (unsigned)(bT - aT) * 8u : 0u;
+      const unsigned nC = k >= 2 && hasC && bC > aC ? (unsigned)(bC - aC) * 8u : 0u;
       const unsigned total = __reduce_add_sync(0xffffffffu, nT + nC);
       const unsigned bar = full0 + 8 * s, dst = sbase + s * Sh::STAGE;
       if (lane == 0) mbar_expect_tx(bar, total);
       __syncwarp();
-      if (nT) bulk_row(dst + (unsigned)((lane * Sh::BW + dT) * (int)sizeof(S)), T + aT, nT, bar);
+      if (nT) bulk_row(dst + (unsigned)((lane * Sh::BW + dT) * 8), T + aT, nT, bar);
       if (nC)
-        bulk_row(dst + Sh::TB + (unsigned)(lane * Sh::CW * (int)sizeof(S)), Ci + aC, nC, bar);
+        bulk_row(dst + Sh::TB + (unsigned)(lane * Sh::CW * 8), Ci + aC, nC, bar);
     }
     if (lane == 0) flags[1] = k;
   } else {
     // ---------------- consumers ----------------
-    const W<C> w = make_w(c0, C(0));
+    const W<double> w = make_w(c0, 0.0);
     // this lane's points of a row: x = xb + lane + 32 i
     unsigned inm = 0u;
 #pragma unroll
@@ -171,18 +173,18 @@ __global__ void __launch_bounds__(32 * 9, 3)
       rowi[j] = warp + j * Sh::CONSUMERS;
       comp[j] = t.r0 + rowi[j] < t.re;
     }
-    C zm[Sh::RPT][P];
+    double zm[Sh::RPT][P];
     bool ok = __all_sync(0xffffffffu, mbar_wait(full0, 0) && mbar_wait(full0 + 8, 0));
     if (!ok) {
       atomicOr(dev_err, IGG_DEV_ERR_TIMEOUT);
       flags[0] = 1;
     } else {
-      const S *Tb = reinterpret_cast<const S *>(smem);
+      const double *Tb = reinterpret_cast<const double *>(smem);
 #pragma unroll
       for (int j = 0; j < Sh::RPT; ++j) {
-        const S *row = Tb + (rowi[j] + 1) * Sh::BW + shT((int)(e0 - usz + (unsigned)(nx * rowi[j])));
+        const double *row = Tb + (rowi[j] + 1) * Sh::BW + shT((int)(e0 - usz + (unsigned)(nx * rowi[j])));
 #pragma unroll
-        for (int i = 0; i < P; ++i) zm[j][i] = Num<S>::cv(row[32 * i]);
+        for (int i = 0; i < P; ++i) zm[j][i] = row[32 * i];
       }
       __syncwarp();
       if (lane == 0) mbar_arrive(empty0);
@@ -215,21 +217,21 @@ __global__ void __launch_bounds__(32 * 9, 3)
         break;
       }
       consumed = k + 2;
-      const S *Tc = reinterpret_cast<const S *>(smem + s * Sh::STAGE);
-      const S *Tn = reinterpret_cast<const S *>(smem + s1 * Sh::STAGE);
-      const S *Cn = reinterpret_cast<const S *>(smem + s1 * Sh::STAGE + Sh::TB);
+      const double *Tc = reinterpret_cast<const double *>(smem + s * Sh::STAGE);
+      const double *Tn = reinterpret_cast<const double *>(smem + s1 * Sh::STAGE);
+      const double *Cn = reinterpret_cast<const double *>(smem + s1 * Sh::STAGE + Sh::TB);
 #pragma unroll
       for (int j = 0; j < Sh::RPT; ++j) {
         const int r = rowi[j];
         const int er = (int)(e + (unsigned)(nx * r));
-        const S *row = Tc + (r + 1) * Sh::BW + shT(er);
-        const S *up = Tc + r * Sh::BW + shT(er - nx);
-        const S *dn = Tc + (r + 2) * Sh::BW + shT(er + nx);
-        const S *zpr = Tn + (r + 1) * Sh::BW + shT((int)((unsigned)er + usz));
-        const S *cir = Cn + r * Sh::CW + shC(er + 1);
-        C c[P], out[P];
+        const double *row = Tc + (r + 1) * Sh::BW + shT(er);
+        const double *up = Tc + r * Sh::BW + shT(er - nx);
+        const double *dn = Tc + (r + 2) * Sh::BW + shT(er + nx);
+        const double *zpr = Tn + (r + 1) * Sh::BW + shT((int)((unsigned)er + usz));
+        const double *cir = Cn + r * Sh::CW + shC(er + 1);
+        double c[P], out[P];
 #pragma unroll
-        for (int i = 0; i < P; ++i) c[i] = Num<S>::cv(row[32 * i]);
+        for (int i = 0; i < P; ++i) c[i] = row[32 * i];
         unsigned okm = (1u << P) - 1u;
         if constexpr (EMU) {
           constexpr int NG = 5 - MODE;
@@ -273,18 +275,17 @@ __global__ void __launch_bounds__(32 * 9, 3)
         } else {
 #pragma unroll
           for (int i = 0; i < P; ++i) {
-            const C xm = Num<S>::cv(row[32 * i - 1]), xp = Num<S>::cv(row[32 * i + 1]);
-            const C ym = Num<S>::cv(up[32 * i]), yp = Num<S>::cv(dn[32 * i]);
-            const C zp = Num<S>::cv(zpr[32 * i]), ci = Num<S>::cv(cir[32 * i]);
-            if constexpr (MODE == 1) out[i] = cell_f64(c[i], xm, xp, ym, yp, zm[j][i], zp, ci, w);
-            else out[i] = cell(c[i], xm, xp, ym, yp, zm[j][i], zp, ci, w);
+            const double xm = row[32 * i - 1], xp = row[32 * i + 1];
+            const double ym = up[32 * i], yp = dn[32 * i];
+            const double zp = zpr[32 * i], ci = cir[32 * i];
+            out[i] = cell_f64(c[i], xm, xp, ym, yp, zm[j][i], zp, ci, w);
           }
         }
         const long long di = t.base + t.xb + lane + (long long)nx * (t.r0 + r) + sz * m;
         if (comp[j]) {
 #pragma unroll
           for (int i = 0; i < P; ++i)
-            if ((inm >> i & 1u) && in_bounds(di + 32 * i, c0.npts)) Num<S>::st(T2 + di + 32 * i, out[i]);
+            if ((inm >> i & 1u) && in_bounds(di + 32 * i, c0.npts)) T2[di + 32 * i] = out[i];
         }
         if constexpr (EMU) {
           // list each 32-point segment of the row with refused points
@@ -329,70 +330,50 @@ __global__ void __launch_bounds__(32 * 9, 3)
   }
 }
 
-template <class S, int MODE>
+template <int MODE>
 cudaError_t prepare_t(int *ctas) {
-  using Sh = RowsShape<S>;
-  cudaError_t e = cudaFuncSetAttribute(k_stencil_rows<S, MODE>,
+  cudaError_t e = cudaFuncSetAttribute(k_stencil_rows<MODE>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, Sh::SMEM);
   if (e == cudaSuccess && ctas)
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas, k_stencil_rows<S, MODE>,
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas, k_stencil_rows<MODE>,
                                                       32 * (Sh::CONSUMERS + 1), Sh::SMEM);
   return e;
 }
 
-template <class S, int MODE>
+template <int MODE>
 cudaError_t launch_t(const TmaTile *tiles, int ntiles, void *T2, const void *T, const void *Ci,
                      int nx, int ny, const Coef &c, unsigned *dev_err, FixBuf fix, cudaStream_t s) {
-  using Sh = RowsShape<S>;
-  return launch_pdl(pdl_on(c.npts), k_stencil_rows<S, MODE>, ntiles, 32 * (Sh::CONSUMERS + 1), Sh::SMEM, s, tiles,
-                    (S *)T2, (const S *)T, (const S *)Ci, nx, ny, c, dev_err, fix.p, fix.cap);
+  return launch_pdl(pdl_on(c.npts), k_stencil_rows<MODE>, ntiles, 32 * (Sh::CONSUMERS + 1), Sh::SMEM, s, tiles,
+                    (double *)T2, (const double *)T, (const double *)Ci, nx, ny, c, dev_err, fix.p, fix.cap);
 }
 
 }  // namespace
 
-int rows_tile_width(igg_dtype dt) {
-  return dt == IGG_F64 ? RowsShape<double>::W
-                       : dt == IGG_F32 ? RowsShape<float>::W : RowsShape<__nv_bfloat16>::W;
-}
-int rows_tile_rows(igg_dtype) { return RowsShape<double>::H; }
+int rows_tile_width() { return Sh::W; }
+int rows_tile_rows() { return Sh::H; }
 
-cudaError_t rows_prepare(igg_dtype dt, int *ctas) {
-  switch (dt) {
-    case IGG_F64: {
-      cudaError_t e = prepare_t<double, 1>(nullptr);
-      if (e == cudaSuccess) e = prepare_t<double, 2>(nullptr);
-      if (e == cudaSuccess) e = prepare_t<double, 4>(nullptr);
-      return e == cudaSuccess ? prepare_t<double, 3>(ctas) : e;
-    }
-    case IGG_F32: return prepare_t<float, 0>(ctas);
-    case IGG_BF16: return prepare_t<__nv_bfloat16, 0>(ctas);
-  }
-  return cudaErrorInvalidValue;
+cudaError_t rows_prepare(int *ctas) {
+  cudaError_t e = prepare_t<1>(nullptr);
+  if (e == cudaSuccess) e = prepare_t<2>(nullptr);
+  if (e == cudaSuccess) e = prepare_t<4>(nullptr);
+  return e == cudaSuccess ? prepare_t<3>(ctas) : e;
 }
 
-cudaError_t launch_stencil_rows(igg_dtype dt, const TmaTile *tiles, int ntiles, void *T2,
-                                const void *T, const void *Ci, int nx, int ny, long long nzt,
-                                const Coef &c, unsigned *dev_err, FixBuf fix, cudaStream_t s) {
+cudaError_t launch_stencil_rows(const TmaTile *tiles, int ntiles, void *T2, const void *T,
+                                const void *Ci, int nx, int ny, long long nzt, const Coef &c,
+                                unsigned *dev_err, FixBuf fix, cudaStream_t s) {
   if (ntiles <= 0) return cudaSuccess;
   Coef cc = c;
   cc.npts = (long long)nx * ny * nzt;
-  switch (dt) {
-    case IGG_F64: {
-      if (!c.f64_emu) return launch_t<double, 1>(tiles, ntiles, T2, T, Ci, nx, ny, cc, dev_err, fix, s);
-      if (!fix.p) return cudaErrorInvalidValue;
-      cudaError_t e;
-      switch (weight_groups(c.wx, c.wy, c.wz)) {
-        case 1: e = launch_t<double, 4>(tiles, ntiles, T2, T, Ci, nx, ny, cc, dev_err, fix, s); break;
-        case 2: e = launch_t<double, 3>(tiles, ntiles, T2, T, Ci, nx, ny, cc, dev_err, fix, s); break;
-        default: e = launch_t<double, 2>(tiles, ntiles, T2, T, Ci, nx, ny, cc, dev_err, fix, s);
-      }
-      return e == cudaSuccess ? launch_fixup(fix, T2, T, Ci, nx, ny, cc, s) : e;
-    }
-    case IGG_F32: return launch_t<float, 0>(tiles, ntiles, T2, T, Ci, nx, ny, cc, dev_err, fix, s);
-    case IGG_BF16:
-      return launch_t<__nv_bfloat16, 0>(tiles, ntiles, T2, T, Ci, nx, ny, cc, dev_err, fix, s);
+  if (!c.f64_emu) return launch_t<1>(tiles, ntiles, T2, T, Ci, nx, ny, cc, dev_err, fix, s);
+  if (!fix.p) return cudaErrorInvalidValue;
+  cudaError_t e;
+  switch (weight_groups(c.wx, c.wy, c.wz)) {
+    case 1: e = launch_t<4>(tiles, ntiles, T2, T, Ci, nx, ny, cc, dev_err, fix, s); break;
+    case 2: e = launch_t<3>(tiles, ntiles, T2, T, Ci, nx, ny, cc, dev_err, fix, s); break;
+    default: e = launch_t<2>(tiles, ntiles, T2, T, Ci, nx, ny, cc, dev_err, fix, s);
   }
-  return cudaErrorInvalidValue;
+  return e == cudaSuccess ? launch_fixup(fix, T2, T, Ci, nx, ny, cc, s) : e;
 }
 
 cudaError_t rows_bounds_flag(unsigned *out, bool clear) { return read_bounds_flag(out, clear); }

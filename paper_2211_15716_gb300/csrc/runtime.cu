@@ -461,16 +461,15 @@ int grid_vec(const igg_grid *g, igg_dtype dt) {
   return (V > 1 && g->n[0] % V == 0) ? V : 1;
 }
 
-// Tiles of one box per subdomain, for the full step.
-// The row-copy kernel takes the full step of the other 3-D grids (rows not a
-// multiple of 16 bytes), down to rows of kRowsMinNx points.
-bool use_rows(const igg_grid *g, int V) {
-  return V == 1 && g->tma_enabled && !low_dim(g) && g->n[0] >= kRowsMinNx;
+// The row-copy kernel takes the full FP64 step of 3-D grids of odd row length,
+// down to rows of kRowsMinNx points (FP32 and BF16: slower there, see rows.cu).
+bool use_rows(const igg_grid *g, int V, igg_dtype dt) {
+  return dt == IGG_F64 && V == 1 && g->tma_enabled && !low_dim(g) && g->n[0] >= kRowsMinNx;
 }
 
-// Key of the full step's tile tables: the vector width, or, for V = 1, 16 +
-// the dtype (the row-copy kernel's tile width depends on it).
-int full_key(const igg_grid *g, int V, igg_dtype dt) { return use_rows(g, V) ? 16 + (int)dt : V; }
+// Key of the full step's tile tables: the vector width, or 16 with the row-copy
+// kernel.
+int full_key(const igg_grid *g, int V, igg_dtype dt) { return use_rows(g, V, dt) ? 16 : V; }
 
 // The full step's TMA tiles of every subdomain. Tile order: for each (z
 // chunk, row block) the tiles of the subdomains that are neighbours in x
@@ -526,13 +525,13 @@ int build_full_tiles(igg_grid *g, int V, igg_dtype dt, TileSet **out) {
   const long long wave2 = 2 * (tma_slots(V) / 3);
   const bool inl = tma && V == 2 && xyt * ((nz - 2 + kInlPlanes - 1) / kInlPlanes) <= wave2;
   if (inl) zbt = choose_zb_tma(xyt, nz - 2, wave2);
-  const bool rows = use_rows(g, V);
+  const bool rows = use_rows(g, V, dt);
   if (tma) {
     full_tma_list(g, V, zbt, Wt, Ht, v.tma);
   } else if (rows) {
-    const int W = rows_tile_width(dt), H = rows_tile_rows(dt);
+    const int W = rows_tile_width(), H = rows_tile_rows();
     int per_sm = 1, sms = 152;
-    cudaError_t e = rows_prepare(dt, &per_sm);
+    cudaError_t e = rows_prepare(&per_sm);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, g->device);
     if (e != cudaSuccess) return cuda_error(e, "row-copy kernel set-up");
     const long long xyt = (long long)((nx - 2 + W - 1) / W) * ((ny - 2 + H - 1) / H) * g->nsub;
@@ -686,7 +685,7 @@ int build_split_tiles(igg_grid *g, const int w[3], int V, SplitTiles **out) {
 cudaError_t launch_tiles(const igg_grid *g, int V, igg_dtype dt, const TileSet &ts, void *T2,
                          const void *T, const void *Ci, const Coef &c, cudaStream_t s) {
   if (ts.tma == TMA_ROWS)
-    return launch_stencil_rows(dt, (const TmaTile *)ts.dev, ts.n, T2, T, Ci, g->n[0], g->n[1],
+    return launch_stencil_rows((const TmaTile *)ts.dev, ts.n, T2, T, Ci, g->n[0], g->n[1],
                                (long long)g->nsub * g->n[2], c, g->dev_err, ts.fix, s);
   if (ts.tma >= 0)
     return launch_stencil_tma(dt, ts.tma, (const TmaTile *)ts.dev, ts.n, T2, T, Ci, g->n[0],

@@ -10,8 +10,9 @@ import synth
 
 pytestmark = pytest.mark.gpu
 
-# 32 points is the shortest row it takes; tiles are 128 points by 8 (FP64) or 16
-# rows; one, two and three weight groups come from the spacings
+# 32 points is the shortest row it takes; FP64 tiles are 128 points by 8
+# rows (the other types take the scalar kernel); one, two and three weight
+# groups come from the spacings
 CASES = [((33, 5, 4), (1, 1, 1)), ((35, 11, 9), (2, 1, 1)), ((127, 10, 6), (1, 2, 1)),
          ((129, 19, 7), (1, 1, 2)), ((131, 18, 5), (2, 2, 1)), ((259, 35, 20), (1, 1, 1)),
          ((31, 9, 6), (2, 1, 1))]
