@@ -83,18 +83,19 @@ __device__ __forceinline__ void ac_put(S *p, S v, const AcSend &a, long long np,
 // 20 KB in flight per SM, short of what the latency of device memory asks for
 // (FP64 launches, bound by the FP64 pipe, only lose issue slots to it): 2x1x2 x
 // 255x193x130, ten steps, 2.71 to 2.59 ms; 2x2x2 x 256^3 FP64, four, 11.28 with-
-// out, 11.62 ms with it.
+// out, 11.62 ms with it. Not where the fields fit in L2: 16 steps of 2x1x2 x 96^3
+// (57 MB) 0.70 ms without, 0.84 with it; of 2x2x1 x 128^3 (134 MB) 1.77 and 1.66.
 constexpr int kAcAhead = 3;
 template <class S>
 __device__ __forceinline__ void ac_ahead(const S *p) {
-  if (sizeof(S) == 4) asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
+  asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
 }
 
 template <class S>
 __global__ void __launch_bounds__(kAcX *kAcY)
     k_acoustic_v(int nx, int ny, int nz, int zchunks, const S *P, S *__restrict__ Vx,
                  S *__restrict__ Vy, S *__restrict__ Vz, const AcW<S> w,
-                 const int *__restrict__ nbr, int ox, int xsend) {
+                 const int *__restrict__ nbr, int ox, int xsend, int ahead) {
   using N = AcNum<S>;
   const int i = blockIdx.x * kAcX + threadIdx.x, j = blockIdx.y * kAcY + threadIdx.y;
   if (i >= nx || j >= ny) return;
@@ -135,11 +136,11 @@ __global__ void __launch_bounds__(kAcX *kAcY)
     // plane k + 1
     const bool nxt = k + 1 < k1;
     S pc1 = S(0), pxm1 = S(0), pym1 = S(0), vx1 = S(0), vy1 = S(0), vz1 = S(0);
-    if (k + kAcAhead < k1) {
-      ac_ahead(Ps + sp * (k + kAcAhead));
-      ac_ahead(Vxs + sx * (k + kAcAhead));
-      ac_ahead(Vys + sy * (k + kAcAhead));
-      ac_ahead(Vzs + sp * (k + kAcAhead));
+    if (sizeof(S) == 4 && k + ahead < k1) {
+      ac_ahead(Ps + sp * (k + ahead));
+      ac_ahead(Vxs + sx * (k + ahead));
+      ac_ahead(Vys + sy * (k + ahead));
+      ac_ahead(Vzs + sp * (k + ahead));
     }
     if (nxt) {
       pc1 = Ps[sp * (k + 1)];
@@ -187,7 +188,7 @@ template <class S>
 __global__ void __launch_bounds__(kAcX *kAcY)
     k_acoustic_p(int nx, int ny, int nz, int zchunks, S *__restrict__ P,
                  const S *Vx, const S *Vy, const S *Vz, const AcW<S> w,
-                 const int *__restrict__ nbr, int ox, int xsend) {
+                 const int *__restrict__ nbr, int ox, int xsend, int ahead) {
   using N = AcNum<S>;
   const int i = blockIdx.x * kAcX + threadIdx.x, j = blockIdx.y * kAcY + threadIdx.y;
   if (i >= nx || j >= ny) return;
@@ -218,11 +219,11 @@ __global__ void __launch_bounds__(kAcX *kAcY)
     // plane k + 1
     const bool nxt = k + 1 < k1;
     S pc1 = S(0), x01 = S(0), x11 = S(0), y01 = S(0), y11 = S(0), vzp1 = S(0);
-    if (k + kAcAhead < k1) {
-      ac_ahead(Ps + sp * (k + kAcAhead));
-      ac_ahead(Vxs + sx * (k + kAcAhead));
-      ac_ahead(Vys + sy * (k + kAcAhead));
-      ac_ahead(Vzs + sp * (k + kAcAhead));
+    if (sizeof(S) == 4 && k + ahead < k1) {
+      ac_ahead(Ps + sp * (k + ahead));
+      ac_ahead(Vxs + sx * (k + ahead));
+      ac_ahead(Vys + sy * (k + ahead));
+      ac_ahead(Vzs + sp * (k + ahead));
     }
     if (nxt) {
       pc1 = Ps[sp * (k + 1)];
@@ -258,11 +259,22 @@ cudaError_t launch_t(int nsub, int nx, int ny, int nz, void *P, void *Vx, void *
   const dim3 grid((nx + kAcX - 1) / kAcX, (ny + kAcY - 1) / kAcY, (unsigned)gz);
   const dim3 block(kAcX, kAcY);
   const AcW<S> w = {(S)c.ax, (S)c.ay, (S)c.az, (S)c.bx, (S)c.by, (S)c.bz, S(1)};
-  cudaError_t e = launch_pdl(true, k_acoustic_v<S>, grid, block, 0, s, nx, ny, nz, zchunks, (const S *)P,
-                             (S *)Vx, (S *)Vy, (S *)Vz, w, c.nbr, c.ox, c.xsend);
+  // FP64: the CTAs of a dependent launch fill the SMs that the one before leaves
+  // room on, and where those are neither idle nor soon drained the FP64 pipes end
+  // up with unequal shares (16 steps, early start against none: 64^3, 32 CTAs,
+  // 547 and 610 us; 2x1x2 x 70x60x64, 192, 1762 and 1022; 2x1x1 x 128^3, 512,
+  // 2137 and 2023; 2x1x2 x 200x160x128, 2240, 6492 and 6590). FP32 launches gain
+  // at every size.
+  const long long ctas = (long long)grid.x * grid.y * grid.z;
+  const bool pdl = sizeof(S) == 4 || ctas <= 152 || ctas > 2 * 4 * 152;
+  // (kAcAhead: fields that stay in L2 only lose issue slots to the prefetches)
+  const long long bytes = 4ll * nsub * nx * ny * nz * (long long)sizeof(S);
+  const int ahead = bytes > (96ll << 20) ? kAcAhead : nz;
+  cudaError_t e = launch_pdl(pdl, k_acoustic_v<S>, grid, block, 0, s, nx, ny, nz, zchunks, (const S *)P,
+                             (S *)Vx, (S *)Vy, (S *)Vz, w, c.nbr, c.ox, c.xsend, ahead);
   if (e != cudaSuccess) return e;
-  return launch_pdl(true, k_acoustic_p<S>, grid, block, 0, s, nx, ny, nz, zchunks, (S *)P, (const S *)Vx,
-                    (const S *)Vy, (const S *)Vz, w, c.nbr, c.ox, c.xsend);
+  return launch_pdl(pdl, k_acoustic_p<S>, grid, block, 0, s, nx, ny, nz, zchunks, (S *)P, (const S *)Vx,
+                    (const S *)Vy, (const S *)Vz, w, c.nbr, c.ox, c.xsend, ahead);
 }
 
 }  // namespace
