@@ -229,6 +229,16 @@ struct FixBuf {
 };
 size_t tma_fix_cap(const TmaTile *tiles, int ntiles);
 inline size_t tma_fix_bytes(size_t cap) { return cap * 16 + 2 * sizeof(unsigned) + 16; }
+// on: the halo cells of T that have a neighbour are not up to date: the launch
+// reads the neighbours' points in their place (the value the halo update would
+// have copied there: plane n_d - o_d of the left, o_d - 1 of the right
+// neighbour in dimension d). nbr as in HaloGather. FP32 and BF16, TMA_WIDE, more
+// than one tile in an x or y with exchanges.
+struct VirtHalo {
+  const int *nbr = nullptr;
+  int on = 0, nz = 0;
+  int o[3] = {0, 0, 0};
+};
 // The fix-up of the launch before it on the stream (c.npts set).
 cudaError_t launch_fixup(FixBuf fix, void *T2, const void *T, const void *Ci, int nx, int ny,
                          const Coef &c, cudaStream_t s);
@@ -247,7 +257,7 @@ cudaError_t launch_stencil_rows(const TmaTile *tiles, int ntiles, void *T2, cons
 cudaError_t launch_stencil_tma(igg_dtype dt, int variant, const TmaTile *tiles, int ntiles,
                                void *T2, const void *T, const void *Ci, int nx, int ny,
                                long long nzt, const Coef &c, unsigned *dev_err,
-                               FixBuf fix, bool inl, cudaStream_t s);
+                               FixBuf fix, bool inl, const VirtHalo &vh, cudaStream_t s);
 
 // Staggered-grid acoustics (acoustic.cu): coefficients dt/(rho dd) of the
 // velocity update and dt K/dd of the pressure update, formed on the host in

@@ -683,13 +683,23 @@ int build_split_tiles(igg_grid *g, const int w[3], int V, SplitTiles **out) {
 }
 
 cudaError_t launch_tiles(const igg_grid *g, int V, igg_dtype dt, const TileSet &ts, void *T2,
-                         const void *T, const void *Ci, const Coef &c, cudaStream_t s) {
+                         const void *T, const void *Ci, const Coef &c, cudaStream_t s,
+                         bool virt = false) {
   if (ts.tma == TMA_ROWS)
     return launch_stencil_rows((const TmaTile *)ts.dev, ts.n, T2, T, Ci, g->n[0], g->n[1],
                                (long long)g->nsub * g->n[2], c, g->dev_err, ts.fix, s);
-  if (ts.tma >= 0)
+  if (ts.tma >= 0) {
+    VirtHalo vh;
+    if (virt) {
+      vh.on = 1;
+      vh.nbr = g->nbr;
+      vh.nz = g->n[2];
+      for (int d = 0; d < 3; ++d) vh.o[d] = g->overlap[d];
+    }
     return launch_stencil_tma(dt, ts.tma, (const TmaTile *)ts.dev, ts.n, T2, T, Ci, g->n[0],
-                              g->n[1], (long long)g->nsub * g->n[2], c, g->dev_err, ts.fix, ts.inl, s);
+                              g->n[1], (long long)g->nsub * g->n[2], c, g->dev_err, ts.fix, ts.inl,
+                              vh, s);
+  }
   if (V > 1) return launch_stencil_vec(dt, (const VTile *)ts.dev, ts.n, T2, T, Ci, c, nullptr, s);
   return launch_stencil(dt, (const Tile *)ts.dev, ts.n, T2, T, Ci, c, nullptr, s);
 }
@@ -868,10 +878,22 @@ cudaEvent_t phase_event(igg_grid *g, cudaStream_t s, int k) {
   return g->pev[i];
 }
 
-// What a step inside igg_run leaves out: its phase events.
+// What a step inside igg_run leaves out: the halo update of its result (no
+// gather), its phase events; virt: T's halo cells are not up to date, the
+// stencil reads the neighbours' points instead.
 struct StepOpt {
-  bool timed = true;
+  bool virt = false, gather = true, timed = true;
 };
+
+// Whether igg_run may leave the halo cells of intermediate states out of date:
+// the full step of an FP32 or BF16 field on the TMA kernel, with exchanges,
+// and more than one tile in x and y where they have them (a tile patches one
+// side of each).
+bool virt_applies(const igg_grid *g, int V, igg_dtype dt) {
+  return dt != IGG_F64 && use_fused_halo(g) && !g->hide_halo && use_tma(g, V) && any_halo(g) &&
+         (g->ncopies[0] == 0 || g->n[0] - 1 > tma_tile_width(dt, TMA_WIDE)) &&
+         (g->ncopies[1] == 0 || g->n[1] - 2 > tma_tile_rows(dt, TMA_WIDE));
+}
 
 // One step of Fig. 1's loop, queued on s: plain (full step, then halo update
 // of T2 on s) or hidden (boundary set + halo on the high-priority stream,
@@ -940,12 +962,12 @@ int enqueue_step(igg_grid *g, const int *widths, void *T2, const void *T, const 
     c.ends = with_halo && any_halo(g) ? 1 : 0;
     {
       NvtxRange r("stencil");
-      e = launch_tiles(g, V, dt, *full, T2, T, Ci, c, s);
+      e = launch_tiles(g, V, dt, *full, T2, T, Ci, c, s, opt.virt);
     }
     if (e != cudaSuccess) return cuda_error(e, "stencil launch");
     if (cudaEvent_t p1 = p0 ? phase_event(g, s, 1) : nullptr)
       if ((e = cudaEventRecord(p1, s)) != cudaSuccess) return cuda_error(e, "record");
-    if (with_halo && any_halo(g)) {
+    if (with_halo && any_halo(g) && opt.gather) {
       NvtxRange r("halo update");
       e = enqueue_halo(g, T2, dtype_size(dt), s);
       if (e != cudaSuccess) return cuda_error(e, "halo launch");
@@ -1395,10 +1417,31 @@ int igg_run(igg_grid *g, int nt, const int widths[3], void *T, void *T2, const v
   };
   // The steps [i0, i1) run as launches of a graph of two steps each, on small
   // grids, where a graph launch costs as much as a step, of up to 16 steps (one
-  // 64^3 FP64 array, 100 steps: 512 us with graphs of two, 326 us of fourteen)
+  // 64^3 FP64 array, 100 steps: 512 us with graphs of two, 326 us of fourteen).
+  //
+  // Where the kernel can read a neighbour's points in place of halo cells
+  // (virt_applies), only the last two steps update the halo (both buffers end
+  // as they would with an update in every step); the first reads the halo cells
+  // that the caller gave. The update's strided x columns touch a sector per
+  // element: 46 to 55 us a step on 2x2x2 x 512x256x256, against 0.48 ms (FP32)
+  // and 0.29 ms (BF16) for the stencil, which loses less than half of that to
+  // the patched tiles: ten steps, FP32 5.26 to 4.94, BF16 3.30 to 3.19 ms. FP64
+  // fields update in every step: their stencil lost as much as the update costs
+  // (10.41 against 10.36 ms), and the fix-up, which reads the stencils again,
+  // more (sign-changing field 14.7 against 12.3 ms).
+  const bool virt = nt >= 4 && virt_applies(g, V, dt);
   StepOpt mid;
   mid.timed = false;
-  const int i0 = 0, i1 = nt - nt % 2;
+  if (virt) {
+    mid.virt = true;
+    mid.gather = false;
+  }
+  const int i0 = virt ? 1 : 0, i1 = virt ? nt - 2 : nt - nt % 2;
+  if (virt) {
+    StepOpt o = mid;
+    o.virt = false;
+    if (int rc = step(0, o, s)) return rc;
+  }
   int i = i0;
   if (i1 - i0 >= 2) {
     // tile tables are allocated before the capture starts
@@ -1418,7 +1461,7 @@ int igg_run(igg_grid *g, int nt, const int widths[3], void *T, void *T2, const v
       const int launches = (pairs + 7) / 8;
       per = pairs / launches;
     }
-    const GraphKey key(T, T2, Ci, (int)dt, (widths ? 1 : 0) + 2 * per,
+    const GraphKey key(T, T2, Ci, (int)dt, (widths ? 1 : 0) + 2 * (virt ? 1 : 0) + 4 * per,
                        widths ? widths[0] : 0, widths ? widths[1] : 0, widths ? widths[2] : 0, c.wx,
                        c.wy, c.wz, c.wc);
     cudaGraphExec_t exec = nullptr;
@@ -1454,7 +1497,14 @@ int igg_run(igg_grid *g, int nt, const int widths[3], void *T, void *T2, const v
   }
   for (; i < i1; ++i)
     if (int rc = step(i, mid, s)) return rc;
-  return nt % 2 ? step(nt - 1, StepOpt(), s) : IGG_OK;
+  if (!virt) return nt % 2 ? step(nt - 1, StepOpt(), s) : IGG_OK;
+  StepOpt o;
+  o.virt = true;
+  o.timed = false;
+  if (int rc = step(nt - 2, o, s)) return rc;
+  o.virt = false;
+  o.timed = nt % 2 != 0;
+  return step(nt - 1, o, s);
 }
 
 int igg_run_host(igg_grid *g, int nt, const int widths[3], void *T_host, const void *Ci_host,

@@ -46,6 +46,16 @@ struct WideShape {
   static constexpr int H = 16;
 };
 
+// The stencil kernel's extra arguments with VirtHalo: the tensor maps of the
+// neighbours' columns (box of one 16-byte vector by BH rows) and rows (BW by 1).
+template <bool VH>
+struct VirtArgs {};
+template <>
+struct VirtArgs<true> {
+  CUtensorMap x, y;
+  VirtHalo h;
+};
+
 template <class S, int LPR_, int H_>
 struct TmaShape {
   static constexpr int V = 16 / (int)sizeof(S);
@@ -62,10 +72,19 @@ struct TmaShape {
   static constexpr int TBA = (TB + 127) / 128 * 128;
   static constexpr int CB = W * H * (int)sizeof(S);     // Ci box bytes
   static constexpr int STAGE = (TBA + CB + 127) / 128 * 128;
+  static constexpr int BARS = NS * STAGE;               // full, empty, land [NS]; flags
+  // FP32 and BF16: halo patches (VirtHalo), two sets: an x column of 16-byte
+  // vectors, a y row
+  static constexpr int PXA = (BH * 16 + 127) / 128 * 128;
+  static constexpr int PYA = (BW * (int)sizeof(S) + 127) / 128 * 128;
+  static constexpr int PATCH = BARS + 128;
   // FP64 (emulated cell): per consumer warp, kFixPend fix-up entries staged
   // before they are appended to the tile set's list
-  static constexpr int PEND = NS * STAGE + 2 * NS * 8 + 64;
-  static constexpr int SMEM = PEND + (sizeof(S) == 8 ? CONSUMERS * 16 * 16 : 0);  // + flags, staging
+  static constexpr int PEND = PATCH;
+  static constexpr int SMEM = PATCH + (sizeof(S) == 8 ? CONSUMERS * (int)kFixPend * 16 : 0);
+  static constexpr int SMEM_VH = PATCH + 2 * (PXA + PYA);
+  static_assert(3 * NS * 8 + 16 <= 128, "barriers and flags");
+  static_assert(3 * (SMEM_VH + 1024) <= 228 * 1024, "three CTAs per SM");
   static_assert(H % ROWS_PER_PASS == 0, "rows per tile");
   static_assert(BW <= 256 && BH <= 256, "TMA box dims");
 };
@@ -280,21 +299,28 @@ __device__ __forceinline__ void emu_fix_rows(const double *Tm, const double *Tc,
 //
 // INL (emulated cell): the warps fix up their rows themselves (emu_fix_rows), a
 // stage is freed a step later (its T plane is m - 1 then), two CTAs per SM.
-template <class S, int LPR_, int H_, bool SWAP, int MODE, bool BATCH = false, bool INL = false>
+//
+// VH (FP32, BF16; not SWAP, BATCH): halo cells with a neighbour are read from the
+// neighbour's planes, columns and rows (VirtHalo).
+template <class S, int LPR_, int H_, bool SWAP, int MODE, bool BATCH = false, bool INL = false,
+          bool VH = false>
 __global__ void __launch_bounds__(32 * 9, INL ? 2 : IGG_TMA_MIN_BLOCKS)
     k_stencil_tma(const __grid_constant__ CUtensorMap mapT, const __grid_constant__ CUtensorMap mapC,
                   const TmaTile *__restrict__ tiles, S *__restrict__ T2, int nx, int ny, Coef c0,
                   unsigned *__restrict__ dev_err, void *__restrict__ fix, size_t fix_cap,
-                  const TmaBatch batch = TmaBatch()) {
+                  const TmaBatch batch, const __grid_constant__ VirtArgs<VH> va) {
   using Sh = TmaShape<S, LPR_, H_>;
   using C = typename Num<S>::C;
   constexpr int V = Sh::V, NS = Sh::NS, LPR = Sh::LPR;
   extern __shared__ __align__(128) unsigned char smem[];
   const unsigned sbase = smem_u32(smem);
-  const unsigned full0 = sbase + NS * Sh::STAGE;
+  const unsigned full0 = sbase + Sh::BARS;
   const unsigned empty0 = full0 + NS * 8;
-  volatile int *flags = reinterpret_cast<volatile int *>(smem + NS * Sh::STAGE + 2 * NS * 8);
-  // flags[0]: abort; flags[1]: loads issued; flags[2]: loads consumed
+  const unsigned land0 = empty0 + NS * 8;  // (patched tiles: the copies' landing)
+  volatile int *flags = reinterpret_cast<volatile int *>(smem + Sh::BARS + 3 * NS * 8);
+  // flags[0]: abort; flags[1]: loads issued; flags[2]: loads consumed;
+  // flags[3]: loads land on land0
+  static_assert(!VH || (sizeof(S) != 8 && !BATCH && !SWAP), "VirtHalo");
 
   FixShared *fs = reinterpret_cast<FixShared *>(smem + Sh::PEND);  // (INL)
   const TmaTile t = tiles[blockIdx.x];
@@ -313,19 +339,120 @@ __global__ void __launch_bounds__(32 * 9, INL ? 2 : IGG_TMA_MIN_BLOCKS)
     for (int s = 0; s < NS; ++s) {
       mbar_init(full0 + 8 * s, 1);
       mbar_init(empty0 + 8 * s, Sh::CONSUMERS);
+      if (VH) mbar_init(land0 + 8 * s, 1);
     }
     flags[0] = 0;
     flags[1] = 0;
     flags[2] = 0;
+    flags[3] = 0;
     if constexpr (INL) fs->segs = fs->pts = 0u;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
   __syncthreads();
 
+  // VirtHalo: the neighbours whose planes this tile's halo cells stand for
+  // (left/right per dimension, -1: none, or the tile does not read that face)
+  int nb[6] = {-1, -1, -1, -1, -1, -1};
+  bool patched = false;
+  if constexpr (VH) {
+    if (warp == Sh::CONSUMERS) {
+      const VirtHalo &vh = va.h;
+      const int *n = vh.nbr + 6 * (t.zoff / vh.nz);
+      if (t.xb == 1) nb[0] = n[0];
+      if (t.xe == nx - 1) nb[1] = n[1];
+      if (t.r0 == 1) nb[2] = n[2];
+      if (t.re == ny - 1) nb[3] = n[3];
+      if (t.m0 == 1) nb[4] = n[4];
+      if (t.m1 == vh.nz - 1) nb[5] = n[5];
+      patched = nb[0] >= 0 || nb[1] >= 0 || nb[2] >= 0 || nb[3] >= 0;
+    }
+  }
+
   if (warp == Sh::CONSUMERS) {
     // ---------------- producer ----------------
-    if (lane == 0) {
+    // the plane, in the stack, of T plane m of this tile
+    auto plane = [&](int m) {
+      if constexpr (VH) {
+        const VirtHalo &vh = va.h;
+        if (m == 0 && nb[4] >= 0) return nb[4] * vh.nz + vh.nz - vh.o[2];
+        if (m == vh.nz - 1 && nb[5] >= 0) return nb[5] * vh.nz + vh.o[2] - 1;
+      }
+      return t.zoff + m;
+    };
+    if constexpr (VH) {
+      if (patched) {
+        const VirtHalo &vh = va.h;
+        // Tiles with halo cells in x or y that stand for a neighbour's points: the
+        // neighbour's column or row comes into a patch set with each box, and the
+        // whole warp writes it over the box's halo cells before it hands the load
+        // to the consumers. Load k + 1 is issued before load k is patched. (One
+        // side per dimension: virt_applies asks for more than one tile.)
+        const int dx = nb[0] >= 0 ? 0 : nb[1] >= 0 ? 1 : -1, dy = nb[2] >= 0 ? 0 : nb[3] >= 0 ? 1 : -1;
+        const unsigned pbytes = (dx >= 0 ? Sh::BH * 16u : 0u) +
+                                (dy >= 0 ? Sh::BW * (unsigned)sizeof(S) : 0u);
+        // the neighbour's sent column and row; the halo cells' places in the box
+        const int px = dx ? vh.o[0] - 1 : nx - vh.o[0], py = dy ? vh.o[1] - 1 : ny - vh.o[1];
+        const int cx = V + (dx ? nx - 1 - t.x0 : 0), ry = dy ? ny - t.r0 : 0;
+        const int subx = dx ? nb[1] : nb[0], suby = dy ? nb[3] : nb[2];
+        if (lane == 0) {
+          pdl_trigger();
+          pdl_wait();
+          flags[3] = 1;
+        }
+        __syncwarp();
+        int k = 0;
+        bool ok = true;
+        for (; k <= K; ++k) {
+          if (k < K) {
+            const int s = k % NS;
+            if (k >= NS)
+              ok = __all_sync(0xffffffffu, mbar_wait(empty0 + 8 * s, ((k / NS) - 1) & 1));
+            if (!ok && lane == 0) atomicOr(dev_err, IGG_DEV_ERR_TIMEOUT);
+            ok = ok && !__any_sync(0xffffffffu, flags[0] != 0);
+            if (!ok) break;
+            if (lane == 0) {
+              const unsigned bar = land0 + 8 * s, dst = sbase + s * Sh::STAGE;
+              const unsigned pat = sbase + Sh::PATCH + (k & 1) * (Sh::PXA + Sh::PYA);
+              const int m = t.m0 - 1 + k;
+              mbar_expect_tx(bar, (k >= 2 ? Sh::TB + Sh::CB : Sh::TB) + pbytes);
+              tma_load_3d(dst, pmT, t.x0 - V, t.r0 - 1, plane(m), bar);
+              if (k >= 2) tma_load_3d(dst + Sh::TBA, pmC, t.x0, t.r0, t.zoff + m - 1, bar);
+              if (dx >= 0) tma_load_3d(pat, &va.x, px / V * V, t.r0 - 1, subx * vh.nz + m, bar);
+              if (dy >= 0) tma_load_3d(pat + Sh::PXA, &va.y, t.x0 - V, py, suby * vh.nz + m, bar);
+            }
+          }
+          if (k > 0) {  // patch load k - 1
+            const int q = (k - 1) % NS;
+            ok = __all_sync(0xffffffffu, mbar_wait(land0 + 8 * q, ((k - 1) / NS) & 1));
+            if (!ok) {
+              if (lane == 0) atomicOr(dev_err, IGG_DEV_ERR_TIMEOUT);
+              if (k < K) ++k;  // (load k is issued)
+              break;
+            }
+            S *box = reinterpret_cast<S *>(smem + q * Sh::STAGE);
+            const unsigned char *pb = smem + Sh::PATCH + ((k - 1) & 1) * (Sh::PXA + Sh::PYA);
+            if (dy >= 0) {
+              const uint4 *src = reinterpret_cast<const uint4 *>(pb + Sh::PXA);
+              uint4 *dst = reinterpret_cast<uint4 *>(box + ry * Sh::BW);
+              for (int i = lane; i < Sh::BW * (int)sizeof(S) / 16; i += 32) dst[i] = src[i];
+              __syncwarp();
+            }
+            if (dx >= 0 && lane < Sh::BH)
+              box[lane * Sh::BW + cx] = reinterpret_cast<const S *>(pb)[lane * V + px % V];
+            // these reads and writes before the next copies into their places
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            __syncwarp();
+            if (lane == 0) mbar_arrive(full0 + 8 * q);
+          }
+        }
+        if (lane == 0) {
+          if (!ok) flags[0] = 1;
+          flags[1] = min(k, K);
+        }
+      }
+    }
+    if (!patched && lane == 0) {
       // the earlier launches complete before the first load, and with it before
       // the consumers' first store
       pdl_trigger();
@@ -346,7 +473,7 @@ __global__ void __launch_bounds__(32 * 9, INL ? 2 : IGG_TMA_MIN_BLOCKS)
         mbar_expect_tx(bar, k >= 2 ? Sh::TB + Sh::CB : Sh::TB);
         const int mT = t.m0 - 1 + k, mC = t.m0 - 2 + k;  // march index of the T / Ci plane
         if (!SWAP) {
-          tma_load_3d(dst, pmT, t.x0 - V, t.r0 - 1, t.zoff + mT, bar);
+          tma_load_3d(dst, pmT, t.x0 - V, t.r0 - 1, plane(mT), bar);
           if (k >= 2) tma_load_3d(dst + Sh::TBA, pmC, t.x0, t.r0, t.zoff + mC, bar);
         } else {
           tma_load_3d(dst, pmT, t.x0 - V, mT, t.zoff + t.r0 - 1, bar);
@@ -539,7 +666,7 @@ __global__ void __launch_bounds__(32 * 9, INL ? 2 : IGG_TMA_MIN_BLOCKS)
   // that no bulk copy writes into this CTA's shared memory after it exits.
   if (threadIdx.x == 0 && flags[0]) {
     for (int k = flags[2]; k < flags[1]; ++k) {
-      if (!mbar_wait(full0 + 8 * (k % NS), (k / NS) & 1)) {
+      if (!mbar_wait((VH && flags[3] ? land0 : full0) + 8 * (k % NS), (k / NS) & 1)) {
         atomicOr(dev_err, IGG_DEV_ERR_DRAIN);
         break;
       }
@@ -724,13 +851,18 @@ cudaError_t prepare_t(int *ctas_per_sm) {
       e = cudaFuncSetAttribute(k_stencil_tma<S, Shp::LPR, Shp::H, SWAP, MODE, false, true>,
                                cudaFuncAttributeMaxDynamicSharedMemorySize, Sh::SMEM);
   }
+  if constexpr (sizeof(S) != 8 && !SWAP) {
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(k_stencil_tma<S, Shp::LPR, Shp::H, SWAP, MODE, false, false, true>,
+                               cudaFuncAttributeMaxDynamicSharedMemorySize, Sh::SMEM_VH);
+  }
   return e;
 }
 
 template <class S, class Shp, bool SWAP, int MODE>
 cudaError_t launch_t(const TmaTile *tiles, int ntiles, void *T2, const void *T, const void *Ci,
                      int nx, int ny, long long nzt, const Coef &c, unsigned *dev_err,
-                     FixBuf fix, bool inl, cudaStream_t s) {
+                     FixBuf fix, bool inl, const VirtHalo &vh, cudaStream_t s) {
   using Sh = TmaShape<S, Shp::LPR, Shp::H>;
   CUtensorMap mT, mC;
   const bool ok = SWAP ? encode<S>(&mT, T, nx, ny, nzt, Sh::BW, 1, Sh::BH) &&
@@ -740,15 +872,29 @@ cudaError_t launch_t(const TmaTile *tiles, int ntiles, void *T2, const void *T, 
   if (!ok) return cudaErrorInvalidValue;
   Coef cc = c;
   cc.npts = (long long)nx * ny * nzt;
+  if (vh.on) {
+    if constexpr (sizeof(S) != 8 && !SWAP) {
+      VirtArgs<true> va;
+      va.h = vh;
+      if (!encode<S>(&va.x, T, nx, ny, nzt, Sh::V, Sh::BH, 1) ||
+          !encode<S>(&va.y, T, nx, ny, nzt, Sh::BW, 1, 1))
+        return cudaErrorInvalidValue;
+      return launch_pdl(pdl_on(cc.npts),
+                        k_stencil_tma<S, Shp::LPR, Shp::H, SWAP, MODE, false, false, true>, ntiles,
+                        32 * (Sh::CONSUMERS + 1), Sh::SMEM_VH, s, mT, mC, tiles, (S *)T2, nx, ny, cc,
+                        dev_err, fix.p, fix.cap, TmaBatch(), va);
+    }
+    return cudaErrorInvalidValue;
+  }
   if constexpr (is_emu(MODE) && !SWAP) {
     if (inl)
       return launch_pdl(true, k_stencil_tma<S, Shp::LPR, Shp::H, SWAP, MODE, false, true>, ntiles,
                         32 * (Sh::CONSUMERS + 1), Sh::SMEM, s, mT, mC, tiles, (S *)T2, nx, ny, cc,
-                        dev_err, fix.p, fix.cap, TmaBatch());
+                        dev_err, fix.p, fix.cap, TmaBatch(), VirtArgs<false>());
   }
   cudaError_t e = launch_pdl(pdl_on(cc.npts), k_stencil_tma<S, Shp::LPR, Shp::H, SWAP, MODE>, ntiles,
                              32 * (Sh::CONSUMERS + 1), Sh::SMEM, s, mT, mC, tiles, (S *)T2, nx, ny,
-                             cc, dev_err, fix.p, fix.cap, TmaBatch());
+                             cc, dev_err, fix.p, fix.cap, TmaBatch(), VirtArgs<false>());
   if (e == cudaSuccess && is_emu(MODE))
     e = launch_fixup_t<emu_groups(MODE)>(fix, T2, T, Ci, nx, ny, cc, s);
   return e;
@@ -780,39 +926,39 @@ cudaError_t prepare_v(int variant, int *ctas) {
 template <class S, bool SWAP>
 cudaError_t launch_m(const TmaTile *tiles, int ntiles, void *T2, const void *T, const void *Ci,
                      int nx, int ny, long long nzt, const Coef &c, unsigned *dev_err,
-                     FixBuf fix, bool inl, cudaStream_t s) {
+                     FixBuf fix, bool inl, const VirtHalo &vh, cudaStream_t s) {
   if constexpr (sizeof(S) == 8) {
     if (c.f64_emu) {
       if (!fix.p) return cudaErrorInvalidValue;
       switch (weight_groups(c.wx, c.wy, c.wz)) {
         case 1:
           return launch_t<S, WideShape<S>, SWAP, emu_mode(1)>(tiles, ntiles, T2, T, Ci, nx, ny,
-                                                              nzt, c, dev_err, fix, inl, s);
+                                                              nzt, c, dev_err, fix, inl, vh, s);
         case 2:
           return launch_t<S, WideShape<S>, SWAP, emu_mode(2)>(tiles, ntiles, T2, T, Ci, nx, ny,
-                                                              nzt, c, dev_err, fix, inl, s);
+                                                              nzt, c, dev_err, fix, inl, vh, s);
         default:
           return launch_t<S, WideShape<S>, SWAP, emu_mode(3)>(tiles, ntiles, T2, T, Ci, nx, ny,
-                                                              nzt, c, dev_err, fix, inl, s);
+                                                              nzt, c, dev_err, fix, inl, vh, s);
       }
     }
     return launch_t<S, WideShape<S>, SWAP, MODE_F64>(tiles, ntiles, T2, T, Ci, nx, ny, nzt, c,
-                                                     dev_err, fix, inl, s);
+                                                     dev_err, fix, inl, vh, s);
   } else {
     return launch_t<S, WideShape<S>, SWAP, MODE_CELL>(tiles, ntiles, T2, T, Ci, nx, ny, nzt, c,
-                                                      dev_err, fix, inl, s);
+                                                      dev_err, fix, inl, vh, s);
   }
 }
 
 template <class S>
 cudaError_t launch_v(int variant, const TmaTile *tiles, int ntiles, void *T2, const void *T,
                      const void *Ci, int nx, int ny, long long nzt, const Coef &c,
-                     unsigned *dev_err, FixBuf fix, bool inl, cudaStream_t s) {
+                     unsigned *dev_err, FixBuf fix, bool inl, const VirtHalo &vh, cudaStream_t s) {
   switch (variant) {
     case TMA_WIDE:
-      return launch_m<S, false>(tiles, ntiles, T2, T, Ci, nx, ny, nzt, c, dev_err, fix, inl, s);
+      return launch_m<S, false>(tiles, ntiles, T2, T, Ci, nx, ny, nzt, c, dev_err, fix, inl, vh, s);
     case TMA_WIDE_SWAP:
-      return launch_m<S, true>(tiles, ntiles, T2, T, Ci, nx, ny, nzt, c, dev_err, fix, inl, s);
+      return launch_m<S, true>(tiles, ntiles, T2, T, Ci, nx, ny, nzt, c, dev_err, fix, inl, vh, s);
   }
   return cudaErrorInvalidValue;
 }
@@ -829,7 +975,7 @@ cudaError_t launch_batch_t(const TmaTile *tiles, int ntiles, void *T2, const Tma
   std::memset(&none, 0, sizeof none);
   return launch_pdl(ntiles <= 4 * 152, k_stencil_tma<S, Shp::LPR, Shp::H, false, MODE, true>, ntiles,
                     32 * (Sh::CONSUMERS + 1), Sh::SMEM, s, none, none, tiles, (S *)T2, 0, 0, Coef(),
-                    dev_err, nullptr, 0, b);
+                    dev_err, nullptr, 0, b, VirtArgs<false>());
 }
 
 template <class S>
@@ -958,18 +1104,18 @@ cudaError_t tma_prepare(igg_dtype dt, int variant, int *ctas_per_sm) {
 cudaError_t launch_stencil_tma(igg_dtype dt, int variant, const TmaTile *tiles, int ntiles,
                                void *T2, const void *T, const void *Ci, int nx, int ny,
                                long long nzt, const Coef &c, unsigned *dev_err,
-                               FixBuf fix, bool inl, cudaStream_t s) {
+                               FixBuf fix, bool inl, const VirtHalo &vh, cudaStream_t s) {
   if (ntiles <= 0) return cudaSuccess;
   switch (dt) {
     case IGG_F64:
-      return launch_v<double>(variant, tiles, ntiles, T2, T, Ci, nx, ny, nzt, c, dev_err, fix, inl,
+      return launch_v<double>(variant, tiles, ntiles, T2, T, Ci, nx, ny, nzt, c, dev_err, fix, inl, vh,
                               s);
     case IGG_F32:
-      return launch_v<float>(variant, tiles, ntiles, T2, T, Ci, nx, ny, nzt, c, dev_err, fix, inl,
+      return launch_v<float>(variant, tiles, ntiles, T2, T, Ci, nx, ny, nzt, c, dev_err, fix, inl, vh,
                              s);
     case IGG_BF16:
       return launch_v<__nv_bfloat16>(variant, tiles, ntiles, T2, T, Ci, nx, ny, nzt, c, dev_err,
-                                     fix, inl, s);
+                                     fix, inl, vh, s);
   }
   return cudaErrorInvalidValue;
 }
