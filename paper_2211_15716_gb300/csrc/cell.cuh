@@ -309,14 +309,16 @@ __device__ __forceinline__ bool emu_spread_d(double tc, const unsigned long long
 // differences (as above, negated differences for negative values included),
 //   bits(T2) = bits(T) + Ci * sum_g w_g G_g
 // for as long as T2 stays in T's binade. Each G_g is split exactly into
-// G_g = Gh 2^23 + Gl with -2^22 <= Gl < 2^22 (Gh = (G_g + 2^22) >> 23).
-// Both halves are read off bits as FP32 numbers with exponent 23 minus
-// 1.5 2^23: Gl from 2^23 + 2^22 + Gl (the low 23 bits of G_g + 2^22), Gh
-// from the integer sum Gh + 0x4B400000, the bits of 1.5 2^23 + Gh, which is
-// exact while -2^22 <= Gh < 2^22, i.e. -2^45 - 2^22 <= G_g < 2^45 - 2^22
-// (the fast path requires it; the subtraction of 1.5 2^23 is an FP32 add on
-// the FMA pipe instead of an integer-to-float conversion). With the weights
-// as float pairs,
+// G_g = Gh 2^23 + Gl with -2^22 <= Gl < 2^22 (Gh = (G_g + 2^22) >> 23). Gl is
+// read off bits as an FP32 number with exponent 23 minus 1.5 2^23 (2^23 + 2^22 +
+// Gl: the low 23 bits of G_g + 2^22); Gh is converted, exactly while
+// |Gh| <= 2^24 (the fast path requires -2^24 <= Gh < 2^24, |G_g| up to 2^47). The
+// conversions run on a pipe that is idle otherwise. Read off bits as well (an
+// FP32 addition instead), Gh is limited to 2^22, which half of the points of a
+// field of short waves exceed: they went through the fix-up launch (2x2x2 x
+// 256x128x128, modes up to 8 about 0, twenty steps: 12.4 ms; now 10.4; 2x2x2 x
+// 512x256x256, smooth, ten steps: 10.43 and 10.40; 2x2x2 x 255x127x129, ten: 1.82
+// and 1.85). With the weights as float pairs,
 // S + C = sum_g w_g G_g is formed from error-free FMA products (2^23 wh) Gh,
 // the small terms (2^23 wl) Gh and wh Gl, and a two-sum of the leading
 // products, to about 2^-46 of sum_g |w_g G_g|. Then
@@ -330,7 +332,7 @@ __device__ __forceinline__ bool emu_spread_d(double tc, const unsigned long long
 // same per-point roundings, so both give the same bits.
 //
 // The fast path applies when the seven values share sign and exponent field
-// E in [180, 2008], every Gh in [-2^22, 2^22), Ci is positive with its exponent in
+// E in [180, 2008], every Gh in [-2^24, 2^24), Ci is positive with its exponent in
 // the FP32 range, |Ci_f C| < 2^22 and T2 (after the correction) keeps T's
 // sign and exponent. With |w| <= 2^40 (the host's condition for the emulated
 // cell) |S| < 2^90, so |S| u is a normal double for every such E. E, and the
@@ -364,15 +366,14 @@ __device__ __forceinline__ void emu2_groups(unsigned long long c, const unsigned
 }
 
 // Integer part of the fast path for one point: the group sums of the bit-
-// pattern second differences, split into the bits gh of the FP32 number
-// 1.5 2^23 + Gh and the bits gm of the FP32 number 1.5 2^23 + Gl. The tests'
-// terms are gathered in o and r: the neighbours share sign and exponent with
-// hc (a high word) when o < 2^20, and every Gh lies in [-2^22, 2^22), i.e. gh
-// in [0x4B000000, 0x4B800000), when r < 2^23 (the centre's own test is
+// pattern second differences, split into the integer gh = Gh and the bits gm of
+// the FP32 number 1.5 2^23 + Gl. The tests' terms are gathered in o and r: the
+// neighbours share sign and exponent with hc (a high word) when o < 2^20, and
+// every Gh lies in [-2^24, 2^24) when r < 2^25 (the centre's own test is
 // emu2_centre_ok). nb: x-, x+, y-, y+, z-, z+.
 template <int NG>
 __device__ __forceinline__ void emu2_int(unsigned long long bc, const unsigned long long *nb,
-                                         unsigned hc, unsigned *gh, unsigned *gm, unsigned &o,
+                                         unsigned hc, int *gh, unsigned *gm, unsigned &o,
                                          unsigned &r) {
 #pragma unroll
   for (int i = 0; i < 6; ++i) o |= (unsigned)(nb[i] >> 32) ^ hc;
@@ -381,9 +382,9 @@ __device__ __forceinline__ void emu2_int(unsigned long long bc, const unsigned l
 #pragma unroll
   for (int g = 0; g < NG; ++g) {
     const unsigned lo = (unsigned)G[g];
-    gh[g] = __funnelshift_r(lo, (unsigned)(G[g] >> 32), 23) + 0x4B400000u;
+    gh[g] = (int)__funnelshift_r(lo, (unsigned)(G[g] >> 32), 23);
     gm[g] = (lo & 0x7FFFFFu) | 0x4B000000u;
-    r |= gh[g] ^ 0x4B000000u;
+    r |= (unsigned)gh[g] + (1u << 24);
   }
 }
 
@@ -448,7 +449,7 @@ __device__ __forceinline__ double emu2_apply(unsigned long long bc, unsigned hc,
 // high word included) and r of emu2_int, Ci positive in the FP32 range, and the
 // correction's range (K = Kr - 1.5 2^23).
 __device__ __forceinline__ bool emu2_ok(unsigned o, unsigned r, double ci, float K) {
-  return o < (1u << 20) && r < (1u << 23) && dhi(ci) - (897u << 20) < (254u << 20) &&
+  return o < (1u << 20) && r < (1u << 25) && dhi(ci) - (897u << 20) < (254u << 20) &&
          fabsf(K) < 4194304.0f;
 }
 
@@ -458,12 +459,13 @@ __device__ __forceinline__ double cell_emu_fast(double tc, const unsigned long l
                                                 double ci, const W<double> &w, bool &ok) {
   const unsigned long long bc = dbits(tc);
   const unsigned hc = (unsigned)(bc >> 32);
-  unsigned gh[NG], gm[NG], o = 0u, r = 0u;
+  int gh[NG];
+  unsigned gm[NG], o = 0u, r = 0u;
   emu2_int<NG>(bc, nb, hc, gh, gm, o, r);
   float fh[NG], fl[NG];
 #pragma unroll
   for (int g = 0; g < NG; ++g) {
-    fh[g] = vadd(__uint_as_float(gh[g]), -kMagic);  // Gh, exact where ok
+    fh[g] = __int2float_rn(gh[g]);  // exact where ok
     fl[g] = __uint_as_float(gm[g]);
   }
   float S, C;
@@ -509,8 +511,10 @@ __device__ __forceinline__ long long emu3_aligned(unsigned long long b, unsigned
   const unsigned long long m =
       (b & 0xFFFFFFFFFFFFFull) | ((unsigned long long)(e != 0u) << 52);
   const unsigned d = min(er - max(e, 1u), 63u);  // m < 2^53: shifts past 53 give 0
-  const unsigned long long q = d ? (m + (1ull << (d - 1u))) >> d : m;
-  return ((b ^ cb) >> 63) ? -(long long)q : (long long)q;
+  // floor(m / 2^d + 1/2), for d = 0 too
+  const unsigned long long q = (((m << 1) >> d) + 1u) >> 1;
+  const unsigned long long n = (unsigned long long)((long long)(b ^ cb) >> 63);
+  return (long long)((q ^ n) - n);
 }
 
 // Integer part of the aligned path: the group sums of the aligned values'
@@ -529,8 +533,8 @@ __device__ __forceinline__ bool emu3_int(unsigned long long bc, const unsigned l
 #pragma unroll
   for (int i = 0; i < 6; ++i) o |= (unsigned)(nb[i] >> 32) ^ (unsigned)(bc >> 32);
   if (o < (1u << 20)) {
-    // all seven share sign and exponent (their differences are too large for the
-    // fast path): the bit patterns differ as the aligned integers do
+    // all seven share sign and exponent (refused by another of the fast path's
+    // tests): the bit patterns differ as the aligned integers do
     emu2_groups<NG>(bc, nb, B, G);
   } else {
     unsigned long long I[6];

@@ -239,7 +239,8 @@ __global__ void __launch_bounds__(32 * 9, 3)
           okm = 0u;
 #pragma unroll
           for (int i2 = 0; i2 < P; i2 += 2) {
-            unsigned gh[2][NG], gm[2][NG], o[2] = {0u, 0u}, rr[2] = {0u, 0u};
+            int gh[2][NG];
+            unsigned gm[2][NG], o[2] = {0u, 0u}, rr[2] = {0u, 0u};
             double ci[2];
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
@@ -253,8 +254,7 @@ __global__ void __launch_bounds__(32 * 9, 3)
             float2 fh[NG], fl[NG];
 #pragma unroll
             for (int g = 0; g < NG; ++g) {
-              fh[g] = vadd(make_float2(__uint_as_float(gh[0][g]), __uint_as_float(gh[1][g])),
-                           vset(-kMagic, float2()));
+              fh[g] = make_float2(__int2float_rn(gh[0][g]), __int2float_rn(gh[1][g]));
               fl[g] = make_float2(__uint_as_float(gm[0][g]), __uint_as_float(gm[1][g]));
             }
             float2 Sv, Cv;
