@@ -316,7 +316,7 @@ __device__ __forceinline__ bool emu_spread_d(double tc, const unsigned long long
 // conversions run on a pipe that is idle otherwise. Read off bits as well (an
 // FP32 addition instead), Gh is limited to 2^22, which half of the points of a
 // field of short waves exceed: they went through the fix-up launch (2x2x2 x
-// 256x128x128, modes up to 8 about 0, twenty steps: 12.4 ms; now 10.4; 2x2x2 x
+// 256x128x128, modes up to 8 about 0, twenty steps: 12.4 against 10.5 ms; 2x2x2 x
 // 512x256x256, smooth, ten steps: 10.43 and 10.40; 2x2x2 x 255x127x129, ten: 1.82
 // and 1.85). With the weights as float pairs,
 // S + C = sum_g w_g G_g is formed from error-free FMA products (2^23 wh) Gh,
@@ -504,17 +504,24 @@ __device__ __forceinline__ double cell_emu_fast(double tc, const unsigned long l
 // largest value, like the roundings of the FP64 cell's differences.
 // It applies when Er lies in [180, 2008] and every |G_g| < 2^47.
 // ---------------------------------------------------------------------------
-// b on the grid of 2^(er-1075), signed relative to the centre (bit pattern cb)
-__device__ __forceinline__ long long emu3_aligned(unsigned long long b, unsigned long long cb,
-                                                  unsigned er) {
-  const unsigned e = (unsigned)(b >> 52) & 0x7FFu;
-  const unsigned long long m =
-      (b & 0xFFFFFFFFFFFFFull) | ((unsigned long long)(e != 0u) << 52);
-  const unsigned d = min(er - max(e, 1u), 63u);  // m < 2^53: shifts past 53 give 0
-  // floor(m / 2^d + 1/2), for d = 0 too
-  const unsigned long long q = (((m << 1) >> d) + 1u) >> 1;
-  const unsigned long long n = (unsigned long long)((long long)(b ^ cb) >> 63);
-  return (long long)((q ^ n) - n);
+// b on the grid of 2^(er-1075), signed relative to the centre (high word hc);
+// er10: er + 10. The significand comes to the top of 64 bits, h is twice the
+// shifted value (0 and subnormals, whose leading bit is not there, are shifted
+// out: er >= 180 where the path applies), and (h + 1) >> 1 rounds to the nearest,
+// halves away from zero for either sign. Seven of these are most of the fix-up
+// launch's work, which the integer pipe bounds (73 % busy): with a masked
+// significand, a conditional rounding shift and a conditional negation (about 24
+// instructions instead of 17) twenty steps of the field above took 10.43 instead
+// of 9.86 ms.
+__device__ __forceinline__ unsigned long long emu3_aligned(unsigned long long b, unsigned hc,
+                                                           unsigned er10) {
+  const unsigned hi = (unsigned)(b >> 32);
+  const unsigned d = er10 - ((hi & 0x7FFFFFFFu) >> 20);  // >= 10
+  const unsigned long long m = (b << 11) | (1ull << 63);
+  unsigned long long h;
+  asm("shr.u64 %0, %1, %2;" : "=l"(h) : "l"(m), "r"(d));  // (64 and more: 0)
+  const long long n = (long long)((int)(hi ^ hc) >> 31);
+  return (unsigned long long)(((long long)h ^ n) + 1 >> 1);
 }
 
 // Integer part of the aligned path: the group sums of the aligned values'
@@ -523,15 +530,16 @@ __device__ __forceinline__ long long emu3_aligned(unsigned long long b, unsigned
 template <int NG>
 __device__ __forceinline__ bool emu3_int(unsigned long long bc, const unsigned long long *nb,
                                          int *gh, unsigned *gm, unsigned &er) {
-  unsigned e = (unsigned)(bc >> 52) & 0x7FFu;
+  const unsigned hc = (unsigned)(bc >> 32);
+  unsigned e = hc & 0x7FFFFFFFu;
 #pragma unroll
-  for (int i = 0; i < 6; ++i) e = max(e, (unsigned)(nb[i] >> 52) & 0x7FFu);
-  er = max(e, 1u);
+  for (int i = 0; i < 6; ++i) e = max(e, (unsigned)(nb[i] >> 32) & 0x7FFFFFFFu);
+  er = e >> 20;
   const unsigned long long B = 1ull << 22;
   unsigned long long G[NG];  // G_g + 2^22
   unsigned o = 0u;
 #pragma unroll
-  for (int i = 0; i < 6; ++i) o |= (unsigned)(nb[i] >> 32) ^ (unsigned)(bc >> 32);
+  for (int i = 0; i < 6; ++i) o |= (unsigned)(nb[i] >> 32) ^ hc;
   if (o < (1u << 20)) {
     // all seven share sign and exponent (refused by another of the fast path's
     // tests): the bit patterns differ as the aligned integers do
@@ -539,8 +547,8 @@ __device__ __forceinline__ bool emu3_int(unsigned long long bc, const unsigned l
   } else {
     unsigned long long I[6];
 #pragma unroll
-    for (int i = 0; i < 6; ++i) I[i] = (unsigned long long)emu3_aligned(nb[i], bc, er);
-    emu2_groups<NG>((unsigned long long)emu3_aligned(bc, bc, er), I, B, G);
+    for (int i = 0; i < 6; ++i) I[i] = emu3_aligned(nb[i], hc, er + 10u);
+    emu2_groups<NG>(emu3_aligned(bc, hc, er + 10u), I, B, G);
   }
   unsigned r = 0u;
 #pragma unroll
