@@ -683,26 +683,28 @@ __global__ void __launch_bounds__(32 * 9, INL ? 2 : IGG_TMA_MIN_BLOCKS)
 // as every kernel: the aligned path for stencils across powers of two or
 // zero, else the FP64 cell). The kernel listed every 32-point row segment
 // with such points (its first point and a bit mask). Each warp takes
-// kFixBatch entries at a time (one per lane of lanes 0..kFixBatch-1). Entries
-// with kFixDense points or more go a lane per point of the segment (contiguous
-// loads); the others' listed points are dealt out to the lanes, 32 at a time,
-// in the order of the entries and their bits, so that lanes are not left idle
-// by sparse masks. The points that need the FP64 cell wait in a queue of the
-// warp until 32 of them are there: its eight FP64 instructions hold the SM's
-// FP64 pipe for 128 cycles however few lanes need them, and where a tenth of
-// the points did, nearly every round had some.
-// On a sign-changing field (2x2x2 x 256x128x128, modes up to 8: 80 % of the
-// points listed, a tenth of them FP64), twenty steps: 14.3 to 12.3 ms with the
-// queue, the dense entries and the aligned path's same-exponent form.
+// kFixBatch entries at a time (one per lane; fewer where the list is short, so
+// that all warps get some: 2x1x2 x 35x60x50, the same modes, forty steps, 1.28 ms,
+// 1.48 with eight always) and writes their points one after the other into a list in shared memory; whenever 32 are there, each lane takes
+// one. So no lane is idle but at the end, and what a segment costs besides its
+// points is a shuffle and a store. Points that need the FP64 cell wait in a queue
+// of the warp until 32 of them are there: its eight FP64 instructions hold the
+// SM's FP64 pipe for 128 cycles however few lanes need them.
+// The integer work of the aligned path bounds the launch where many points are
+// listed (2x2x2 x 256x128x128, modes up to 8 about 0: half of them), the latency
+// of its loads where few are. Twenty steps of that field: points dealt to the
+// lanes from batches of four entries by their rank, or a lane per point of the
+// segment for entries of 16 and more, 9.86 ms; with the list 8.59. (Batches of 4
+// and 16 entries 8.56 and 8.66; ten steps of 2x2x2 x 512x256x256, smooth, 10.40
+// before, 10.37 with 8, 10.38 with 4 and 16.)
 // Each block adds its segments and points to the list's totals; the last
 // block to finish resets the list.
-constexpr unsigned kFixBatch = 4;
-constexpr int kFixDense = 16;
+constexpr unsigned kFixBatch = 8;
 template <int NG>
 __global__ void __launch_bounds__(256)
     k_fixup_f64(void *fix, size_t cap, double *T2, const double *T, const double *Ci, int nx, int ny,
                 Coef c0) {
-  __shared__ long long queue[8][64];
+  __shared__ long long queue[8][64], list[8][64];
   pdl_trigger();
   pdl_wait();
   const FixList fl = fix_list(fix, cap);
@@ -734,83 +736,63 @@ __global__ void __launch_bounds__(256)
     }
     __syncwarp();
   };
-  for (unsigned b = gw * kFixBatch; b < count; b += warps * kFixBatch) {
-    FixEntry en = {};
-    if (lane < (int)kFixBatch && b + lane < count) en = fl.e[b + lane];
-    segs += __popc(__ballot_sync(0xffffffffu, en.bits != 0u));
-    pts += __reduce_add_sync(0xffffffffu, (unsigned)__popc(en.bits));
-    // one point per lane, the point at p where `on`
-    auto round = [&](bool on, long long p) {
-      bool f64 = false;
-      if (on && in_bounds(p - sz, c0.npts) && in_bounds(p + sz, c0.npts)) {
-        double tn[6];
-        stencil(p, tn);
-        const double tc = T[p], ci = Ci[p];
-        unsigned long long nb[6];
-#pragma unroll
-        for (int i = 0; i < 6; ++i) nb[i] = dbits(tn[i]);
-        bool ok;
-        const double v = cell_emu_aligned<NG>(tc, nb, ci, w, ok);
-        if (ok) T2[p] = v;
-        f64 = !ok;
+  long long *lst = list[threadIdx.x >> 5];
+  unsigned nlst = 0u;             // warp-uniform, at most 63
+  unsigned next = 0u, have = 0u;  // of the batch's entries
+  FixEntry en = {};
+  const unsigned batch = min(kFixBatch, (count + warps - 1u) / warps);
+  for (unsigned b = gw * batch;;) {
+    // 32 points into the list
+    while (nlst < 32u) {
+      if (next == have) {
+        if (b >= count) break;
+        next = 0u;
+        have = min(batch, count - b);
+        en.bits = 0u;
+        if ((unsigned)lane < have) en = fl.e[b + lane];
+        b += warps * batch;
+        segs += __popc(__ballot_sync(0xffffffffu, en.bits != 0u));
+        pts += __reduce_add_sync(0xffffffffu, (unsigned)__popc(en.bits));
       }
-      const unsigned m = __ballot_sync(0xffffffffu, f64);
-      if (m) {
-        if (f64) que[nque + __popc(m & ((1u << lane) - 1u))] = p;
-        nque += __popc(m);
-        if (nque >= 32u) {
-          run_queue(32u);
-          nque -= 32u;
-          if ((unsigned)lane < nque) que[lane] = que[32 + lane];
-          __syncwarp();  // the moved entries before the next ones
-        }
+      const unsigned bits = __shfl_sync(0xffffffffu, en.bits, next);
+      const long long p0 = __shfl_sync(0xffffffffu, en.p, next);
+      if (bits >> lane & 1u) lst[nlst + __popc(bits & ((1u << lane) - 1u))] = p0 + lane;
+      nlst += __popc(bits);
+      ++next;
+    }
+    if (nlst == 0u) break;
+    __syncwarp();
+    const bool on = (unsigned)lane < nlst;
+    const long long p = on ? lst[lane] : 0;
+    nlst -= min(nlst, 32u);
+    const bool mv = (unsigned)lane < nlst;
+    const long long pn = mv ? lst[32 + lane] : 0;
+    __syncwarp();  // (the list is read before it is written again)
+    if (mv) lst[lane] = pn;
+    __syncwarp();
+    bool f64 = false;
+    if (on && in_bounds(p - sz, c0.npts) && in_bounds(p + sz, c0.npts)) {
+      double tn[6];
+      stencil(p, tn);
+      const double tc = T[p], ci = Ci[p];
+      unsigned long long nb[6];
+#pragma unroll
+      for (int i = 0; i < 6; ++i) nb[i] = dbits(tn[i]);
+      bool ok;
+      const double v = cell_emu_aligned<NG>(tc, nb, ci, w, ok);
+      if (ok) T2[p] = v;
+      f64 = !ok;
+    }
+    const unsigned m = __ballot_sync(0xffffffffu, f64);
+    if (m) {
+      if (f64) que[nque + __popc(m & ((1u << lane) - 1u))] = p;
+      nque += __popc(m);
+      if (nque >= 32u) {
+        run_queue(32u);
+        nque -= 32u;
+        if ((unsigned)lane < nque) que[lane] = que[32 + lane];
+        __syncwarp();  // the moved entries before the next ones
       }
-    };
-    // dense entries (kFixDense points and more): a lane per point of the segment,
-    // its loads and stores contiguous, without dealing
-    unsigned dense = __ballot_sync(0xffffffffu, __popc(en.bits) >= kFixDense);
-    while (dense) {
-      const int q = __ffs(dense) - 1;
-      dense &= dense - 1u;
-      const unsigned bits = __shfl_sync(0xffffffffu, en.bits, q);
-      const long long p0 = __shfl_sync(0xffffffffu, en.p, q);
-      round((bits >> lane & 1u) != 0u, p0 + lane);
-    }
-    if (__popc(en.bits) >= kFixDense) en.bits = 0u;
-    // the others: inclusive prefix of the entries' point counts over lanes
-    // 0..kFixBatch-1
-    unsigned pre = __popc(en.bits);
-#pragma unroll
-    for (unsigned d = 1; d < kFixBatch; d <<= 1) {
-      const unsigned v = __shfl_up_sync(0xffffffffu, pre, d);
-      if ((unsigned)lane >= d) pre += v;
-    }
-    const unsigned total = __shfl_sync(0xffffffffu, pre, kFixBatch - 1);
-    if (total == 0u) continue;
-    unsigned pk[kFixBatch], bk[kFixBatch];
-    long long qk[kFixBatch];
-#pragma unroll
-    for (unsigned q = 0; q < kFixBatch; ++q) {
-      pk[q] = __shfl_sync(0xffffffffu, pre, q);
-      bk[q] = __shfl_sync(0xffffffffu, en.bits, q);
-      qk[q] = __shfl_sync(0xffffffffu, en.p, q);
-    }
-    for (unsigned r = 0; r < total; r += 32u) {
-      const unsigned rank = min(r + lane, total - 1u);
-      // the entry holding the point of this rank and the point's bit
-      unsigned q = 0u;
-#pragma unroll
-      for (unsigned k = 0; k + 1 < kFixBatch; ++k) q += rank >= pk[k] ? 1u : 0u;
-      unsigned bits = bk[0], excl = 0u;
-      long long p0 = qk[0];
-#pragma unroll
-      for (unsigned k = 1; k < kFixBatch; ++k)
-        if (q == k) {
-          bits = bk[k];
-          excl = pk[k - 1];
-          p0 = qk[k];
-        }
-      round(r + lane < total, p0 + __fns(bits, 0u, (int)(rank - excl + 1u)));
     }
   }
   run_queue(nque);
