@@ -93,7 +93,11 @@ template <class S>
 __device__ __forceinline__ void lds_vec(const S *p, Vec<S> &o) {
   unpack(*reinterpret_cast<const uint4 *>(p), o);
 }
-constexpr int kFixupBlocks = 8 * 152;
+// Fix-up blocks: one wave, five per SM (48 registers). Against 8 x 152, ten steps
+// of 2x2x2 x 512x256x256 10.37 and 10.33 ms, of 2x2x2 x 255x127x129 1.857 and
+// 1.814, 48 steps of the misfit gradient at 256^3 20.60 and 20.23, many points
+// listed (k_fixup_f64's field) 8.56 both; 4 x 152: 8.74 there, the others equal.
+constexpr int kFixupBlocks = 5 * 152;
 
 // bit i of x (i < 16) to bit 2i
 __device__ __forceinline__ unsigned spread16(unsigned x) {
@@ -685,11 +689,12 @@ __global__ void __launch_bounds__(32 * 9, INL ? 2 : IGG_TMA_MIN_BLOCKS)
 // with such points (its first point and a bit mask). Each warp takes
 // kFixBatch entries at a time (one per lane; fewer where the list is short, so
 // that all warps get some: 2x1x2 x 35x60x50, the same modes, forty steps, 1.28 ms,
-// 1.48 with eight always) and writes their points one after the other into a list in shared memory; whenever 32 are there, each lane takes
-// one. So no lane is idle but at the end, and what a segment costs besides its
-// points is a shuffle and a store. Points that need the FP64 cell wait in a queue
-// of the warp until 32 of them are there: its eight FP64 instructions hold the
-// SM's FP64 pipe for 128 cycles however few lanes need them.
+// 1.48 with eight always) and writes their points one after the other into a
+// list in shared memory; whenever 32 are there, each lane takes one. So no lane
+// is idle but at the end, and a segment costs a shuffle and a store besides its
+// points. Points that need the FP64 cell wait in a queue of the warp until 32 of
+// them are there: its eight FP64 instructions hold the SM's FP64 pipe for 128
+// cycles however few lanes need them.
 // The integer work of the aligned path bounds the launch where many points are
 // listed (2x2x2 x 256x128x128, modes up to 8 about 0: half of them), the latency
 // of its loads where few are. Twenty steps of that field: points dealt to the
@@ -701,7 +706,7 @@ __global__ void __launch_bounds__(32 * 9, INL ? 2 : IGG_TMA_MIN_BLOCKS)
 // block to finish resets the list.
 constexpr unsigned kFixBatch = 8;
 template <int NG>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, 5)
     k_fixup_f64(void *fix, size_t cap, double *T2, const double *T, const double *Ci, int nx, int ny,
                 Coef c0) {
   __shared__ long long queue[8][64], list[8][64];
