@@ -312,9 +312,9 @@ __device__ __forceinline__ bool emu_spread_d(double tc, const unsigned long long
 // G_g = Gh 2^23 + Gl with -2^22 <= Gl < 2^22 (Gh = (G_g + 2^22) >> 23). Gl is
 // read off bits as an FP32 number with exponent 23 minus 1.5 2^23 (2^23 + 2^22 +
 // Gl: the low 23 bits of G_g + 2^22); Gh is converted, exactly while
-// |Gh| <= 2^24 (the fast path requires -2^24 <= Gh < 2^24, |G_g| up to 2^47). The
-// conversions run on a pipe that is idle otherwise. Read off bits as well (an
-// FP32 addition instead), Gh is limited to 2^22, which half of the points of a
+// |Gh| <= 2^24 (the fast path requires -2^24 <= Gh < 2^24, |G_g| up to 2^47).
+// Read off bits as well (an integer addition in place of the conversion, and an
+// FP32 addition), Gh is limited to 2^22, which half of the points of a
 // field of short waves exceed: they went through the fix-up launch (2x2x2 x
 // 256x128x128, modes up to 8 about 0, twenty steps: 12.4 against 10.5 ms; 2x2x2 x
 // 512x256x256, smooth, ten steps: 10.43 and 10.40; 2x2x2 x 255x127x129, ten: 1.82
