@@ -1,7 +1,8 @@
 // Row-copy stencil kernel: the full FP64 step on 3-D grids of odd row length
 // (255 or 127 points, say), whose rows are not a multiple of 16 bytes: no tensor
 // map takes them (a pitch is a multiple of 16 bytes), and they start at either
-// alignment.
+// alignment. T and Ci themselves start on 16 bytes (use_rows, runtime.cu): a
+// copy's 16-byte boundary is found from the element index.
 //
 // What bounds it: with plain loads, one point per thread and step in flight, it
 // was the latency of the loads (2x2x2 x 255x127x129 FP64, ten steps: 2.57 ms,

@@ -462,14 +462,20 @@ int grid_vec(const igg_grid *g, igg_dtype dt) {
 }
 
 // The row-copy kernel takes the full FP64 step of 3-D grids of odd row length,
-// down to rows of kRowsMinNx points (FP32 and BF16: slower there, see rows.cu).
-bool use_rows(const igg_grid *g, int V, igg_dtype dt) {
-  return dt == IGG_F64 && V == 1 && g->tma_enabled && !low_dim(g) && g->n[0] >= kRowsMinNx;
+// down to rows of kRowsMinNx points (FP32 and BF16: slower there, see rows.cu),
+// whose T and Ci start on 16 bytes: its bulk copies start on the 16-byte
+// boundaries that it counts from there. The caller's fields do (check_field);
+// of the states inside the checkpointed drivers' buffers every other one starts
+// 8 bytes off where the grid has an odd number of points, and a step from such
+// a state takes the scalar kernel (the same bits).
+bool use_rows(const igg_grid *g, int V, igg_dtype dt, const void *T, const void *Ci) {
+  return dt == IGG_F64 && V == 1 && g->tma_enabled && !low_dim(g) && g->n[0] >= kRowsMinNx &&
+         aligned16(T) && aligned16(Ci);
 }
 
 // Key of the full step's tile tables: the vector width, or 16 with the row-copy
 // kernel.
-int full_key(const igg_grid *g, int V, igg_dtype dt) { return use_rows(g, V, dt) ? 16 : V; }
+int full_key(int V, bool rows) { return rows ? 16 : V; }
 
 // The full step's TMA tiles of every subdomain. Tile order: for each (z
 // chunk, row block) the tiles of the subdomains that are neighbours in x
@@ -502,8 +508,9 @@ bool touches_faces(const igg_grid *g, const TmaTile &t) {
          (ex[2] && side(t.m0, t.m1, g->n[2], g->overlap[2]));
 }
 
-int build_full_tiles(igg_grid *g, int V, igg_dtype dt, TileSet **out) {
-  const int key = full_key(g, V, dt);
+// The full step's tile set; rows: of the row-copy kernel (use_rows).
+int build_full_tiles(igg_grid *g, int V, igg_dtype dt, bool rows, TileSet **out) {
+  const int key = full_key(V, rows);
   auto it = g->full.find(key);
   if (it != g->full.end()) {
     *out = &it->second;
@@ -525,7 +532,11 @@ int build_full_tiles(igg_grid *g, int V, igg_dtype dt, TileSet **out) {
   const long long wave2 = 2 * (tma_slots(V) / 3);
   const bool inl = tma && V == 2 && xyt * ((nz - 2 + kInlPlanes - 1) / kInlPlanes) <= wave2;
   if (inl) zbt = choose_zb_tma(xyt, nz - 2, wave2);
-  const bool rows = use_rows(g, V, dt);
+  // (a driver captured into a graph must find both of its sets: no allocation there)
+  if (rows && (g->nsub * g->nloc) % 2 != 0) {
+    TileSet *scalar = nullptr;
+    if (int rc = build_full_tiles(g, V, dt, false, &scalar)) return rc;
+  }
   if (tma) {
     full_tma_list(g, V, zbt, Wt, Ht, v.tma);
   } else if (rows) {
@@ -958,7 +969,7 @@ int enqueue_step(igg_grid *g, const int *widths, void *T2, const void *T, const 
   }
   if (!widths) {
     TileSet *full = nullptr;
-    if (int rc = build_full_tiles(g, V, dt, &full)) return rc;
+    if (int rc = build_full_tiles(g, V, dt, use_rows(g, V, dt, T, Ci), &full)) return rc;
     c.ends = with_halo && any_halo(g) ? 1 : 0;
     {
       NvtxRange r("stencil");
@@ -1453,7 +1464,7 @@ int igg_run(igg_grid *g, int nt, const int widths[3], void *T, void *T2, const v
       if (int rc = build_part_tiles(g, V, &pt)) return rc;
     } else {
       TileSet *full = nullptr;
-      if (int rc = build_full_tiles(g, V, dt, &full)) return rc;
+      if (int rc = build_full_tiles(g, V, dt, use_rows(g, V, dt, T, Ci), &full)) return rc;
     }
     const int pairs = (i1 - i0) / 2;
     int per = 1;  // pairs of steps in the graph
