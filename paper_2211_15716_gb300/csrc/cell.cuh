@@ -519,7 +519,11 @@ __device__ __forceinline__ unsigned long long emu3_aligned(unsigned long long b,
   const unsigned d = er10 - ((hi & 0x7FFFFFFFu) >> 20);  // >= 10
   const unsigned long long m = (b << 11) | (1ull << 63);
   unsigned long long h;
+#ifdef __CUDA_ARCH__
   asm("shr.u64 %0, %1, %2;" : "=l"(h) : "l"(m), "r"(d));  // (64 and more: 0)
+#else
+  h = d < 64u ? m >> d : 0ull;
+#endif
   const long long n = (long long)((int)(hi ^ hc) >> 31);
   return (unsigned long long)(((long long)h ^ n) + 1 >> 1);
 }
@@ -553,12 +557,12 @@ __device__ __forceinline__ bool emu3_int(unsigned long long bc, const unsigned l
   unsigned r = 0u;
 #pragma unroll
   for (int g = 0; g < NG; ++g) {
-    const unsigned lo = (unsigned)G[g];
-    gh[g] = (int)__funnelshift_r(lo, (unsigned)((unsigned long long)G[g] >> 32), 23);
+    const unsigned lo = (unsigned)G[g], hi = (unsigned)(G[g] >> 32);
+    gh[g] = (int)__funnelshift_r(lo, hi, 23);
     gm[g] = (lo & 0x7FFFFFu) | 0x4B000000u;
-    r |= (unsigned)gh[g] + (1u << 24);
+    r |= hi + (1u << 15);
   }
-  return er - 180u <= 1828u && r < (1u << 25);
+  return er - 180u <= 1828u && r < (1u << 16);
 }
 
 // The aligned path for one point; ok tells whether it applies.
