@@ -311,14 +311,16 @@ __device__ __forceinline__ bool emu_spread_d(double tc, const unsigned long long
 // for as long as T2 stays in T's binade. Each G_g is split exactly into
 // G_g = Gh 2^23 + Gl with -2^22 <= Gl < 2^22 (Gh = (G_g + 2^22) >> 23). Gl is
 // read off bits as an FP32 number with exponent 23 minus 1.5 2^23 (2^23 + 2^22 +
-// Gl: the low 23 bits of G_g + 2^22); Gh is converted, exactly while
-// |Gh| <= 2^24 (the fast path requires -2^24 <= Gh < 2^24, |G_g| up to 2^47).
-// Read off bits as well (an integer addition in place of the conversion, and an
-// FP32 addition), Gh is limited to 2^22, which half of the points of a
-// field of short waves exceed: they went through the fix-up launch (2x2x2 x
-// 256x128x128, modes up to 8 about 0, twenty steps: 12.4 against 10.5 ms; 2x2x2 x
-// 512x256x256, smooth, ten steps: 10.43 and 10.40; 2x2x2 x 255x127x129, ten: 1.82
-// and 1.85). With the weights as float pairs,
+// Gl: the low 23 bits of G_g + 2^22); Gh is converted, exactly. The fast path
+// requires -2^22 <= Gh < 2^22, |G_g| up to 2^45: C grows with G_g, and with it
+// what the correction below loses by taking 24 bits of Ci, at the weights of a
+// stable step an eighth of an ulp at 2^45. Taken up to 2^47, the largest error
+// over stencils of one binade was 1.15, 1.24 and 1.30 ulps (one, two and three
+// weight groups) instead of 1.06, 1.13 and 1.19. The points in between, a third of
+// a field of short waves, take the aligned path, which multiplies by all of Ci,
+// through the fix-up launch: 2x2x2 x 256x128x128, modes up to 8 about 0, twenty
+// steps 11.87 instead of 8.83 ms.
+// With the weights as float pairs,
 // S + C = sum_g w_g G_g is formed from error-free FMA products (2^23 wh) Gh,
 // the small terms (2^23 wl) Gh and wh Gl, and a two-sum of the leading
 // products, to about 2^-46 of sum_g |w_g G_g|. Then
@@ -332,7 +334,7 @@ __device__ __forceinline__ bool emu_spread_d(double tc, const unsigned long long
 // same per-point roundings, so both give the same bits.
 //
 // The fast path applies when the seven values share sign and exponent field
-// E in [180, 2008], every Gh in [-2^24, 2^24), Ci is positive with its exponent in
+// E in [180, 2008], every Gh in [-2^22, 2^22), Ci is positive with its exponent in
 // the FP32 range, |Ci_f C| < 2^22 and T2 (after the correction) keeps T's
 // sign and exponent. With |w| <= 2^40 (the host's condition for the emulated
 // cell) |S| < 2^90, so |S| u is a normal double for every such E. E, and the
@@ -369,7 +371,7 @@ __device__ __forceinline__ void emu2_groups(unsigned long long c, const unsigned
 // pattern second differences, split into the integer gh = Gh and the bits gm of
 // the FP32 number 1.5 2^23 + Gl. The tests' terms are gathered in o and r: the
 // neighbours share sign and exponent with hc (a high word) when o < 2^20, and
-// every Gh lies in [-2^24, 2^24) when r < 2^25 (the centre's own test is
+// every Gh lies in [-2^22, 2^22) when r < 2^23 (the centre's own test is
 // emu2_centre_ok). nb: x-, x+, y-, y+, z-, z+.
 template <int NG>
 __device__ __forceinline__ void emu2_int(unsigned long long bc, const unsigned long long *nb,
@@ -384,7 +386,7 @@ __device__ __forceinline__ void emu2_int(unsigned long long bc, const unsigned l
     const unsigned lo = (unsigned)G[g];
     gh[g] = (int)__funnelshift_r(lo, (unsigned)(G[g] >> 32), 23);
     gm[g] = (lo & 0x7FFFFFu) | 0x4B000000u;
-    r |= (unsigned)gh[g] + (1u << 24);
+    r |= (unsigned)gh[g] + (1u << 22);
   }
 }
 
@@ -449,7 +451,7 @@ __device__ __forceinline__ double emu2_apply(unsigned long long bc, unsigned hc,
 // high word included) and r of emu2_int, Ci positive in the FP32 range, and the
 // correction's range (K = Kr - 1.5 2^23).
 __device__ __forceinline__ bool emu2_ok(unsigned o, unsigned r, double ci, float K) {
-  return o < (1u << 20) && r < (1u << 25) && dhi(ci) - (897u << 20) < (254u << 20) &&
+  return o < (1u << 20) && r < (1u << 23) && dhi(ci) - (897u << 20) < (254u << 20) &&
          fabsf(K) < 4194304.0f;
 }
 

@@ -90,5 +90,8 @@ def test_error_and_range(cells, kind, ng):
         # half an ulp of the weights' roundings; 2^-44 of Ci sum |w d2|
         bound = Fr(7, 2) * u + Fr(2) ** -44 * c * sum(a * abs(b) for a, b in zip(wr, d2))
         assert abs(Fr(float(out[i])) - exact) <= bound, (i, path[i], s)
-        if path[i] < 2:  # (the rounded values' sum is within 6 of the exact one)
+        if path[i] == 0:
+            # the correction's Ci of 24 bits costs an eighth of an ulp at 2^45
+            assert max(abs(g) for g in _group_sums(s, u, ng)) <= 2 ** 45 + 2 ** 22, (i, s)
+        elif path[i] == 1:  # (the rounded values' sum is within 6 of the exact one)
             assert max(abs(g) for g in _group_sums(s, u, ng)) <= 2 ** 47 + 2 ** 22 + 6, (i, path[i], s)
