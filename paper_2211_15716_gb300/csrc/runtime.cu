@@ -244,7 +244,13 @@ igg_dtype dtype_of_vec(int V) { return V == 2 ? IGG_F64 : V == 4 ? IGG_F32 : IGG
 
 // z depth of TMA tiles: each tile loads two extra planes of T and of Ci, so
 // deeper is cheaper, but the tile count should fill whole waves of resident
-// CTAs; minimise (extra-plane cost) / (wave efficiency).
+// CTAs; minimise (extra-plane cost) / (wave efficiency). At most 48 planes: where
+// the tiles fill many waves at any depth, deeper ones were chosen for the few
+// planes they save, but resident tiles that march through more planes drift
+// apart, and the rows that neighbours share leave L2 between them. Ten steps,
+// 128 planes (64 with FP32) and 48: 1024^3 FP64 39.2 and 38.0 ms (at 32 and 64
+// planes 37.0 and 37.7 where 48 took 37.3), FP32 19.8 and 19.5, 384^3 FP64 2.32 and
+// 2.18, FP32 1.21 and 1.14, 2x2x1 x 1024x512x256 FP32 9.81 and 9.56.
 int choose_zb_tma(long long xy_tiles, int zext, long long slots) {
   // A box that leaves slots empty even at the smallest depth below (a small
   // grid): the steps are bound by the latency of a tile's march, so as many
@@ -253,9 +259,9 @@ int choose_zb_tma(long long xy_tiles, int zext, long long slots) {
     const long long chunks = std::max<long long>(1, slots / xy_tiles);
     return (int)std::max<long long>(1, (zext + chunks - 1) / chunks);
   }
-  int best = std::min(64, zext);
+  int best = std::min(48, zext);
   double best_cost = 1e30;
-  for (int zb : {16, 24, 32, 40, 48, 64, 96, 128}) {
+  for (int zb : {16, 24, 32, 40, 48}) {
     const int z = std::min(zb, zext);
     const long long nt = xy_tiles * ((zext + z - 1) / z);
     const long long waves = (nt + slots - 1) / slots;
