@@ -301,8 +301,8 @@ int igg_step_hidden(igg_grid *grid, const int widths[3], void *T2,
 /* Fig. 1's time loop: nt times { step (hidden when widths != NULL, else
  * plain step then halo update) of T2 from T; swap T and T2 }. The loop is
  * captured once into a CUDA graph (two steps per graph launch, up to 16 on
- * small grids) and cached on the grid for the same pointers, dtype, widths and
- * coefficients. FP32 and BF16 grids may leave the halo cells of intermediate
+ * small grids) and cached on the grid (the 64 used last) for the same pointers,
+ * dtype, widths and coefficients. FP32 and BF16 grids may leave the halo cells of intermediate
  * states out of date (the step then reads the neighbours' points): T and T2
  * end as with an update in every step.
  * T2 must hold a copy of T's boundary values on entry (Fig. 1 T2 =

@@ -398,7 +398,12 @@ struct igg_grid {
     int ncopies[3] = {0, 0, 0};
   };
   std::map<std::array<int, 3>, Tables> staggered;
-  std::map<GraphKey, cudaGraphExec_t> graphs;
+  struct Graph {
+    cudaGraphExec_t exec;
+    unsigned long long used;  // of graph_uses, at its last use
+  };
+  std::map<GraphKey, Graph> graphs;  // of igg_run, at most kMaxGraphs
+  unsigned long long graph_uses = 0;
   unsigned *dev_err = nullptr;  // device error word of the pipelined kernels
   int *nbr = nullptr;           // device copy of left/right per subdomain and dimension
   bool tma_enabled = true;      // TMA kernel for the regular boxes when available
@@ -1024,6 +1029,45 @@ int enqueue_step(igg_grid *g, const int *widths, void *T2, const void *T, const 
   return IGG_OK;
 }
 
+// The graph of n steps (step(k) queues the k-th on g->cap) kept under key,
+// captured on first use. The cache is bounded: the least recently used graph
+// goes first. (Runs of different numbers of steps on the same fields of a small
+// grid need up to eight graphs, with the buffers swapped as many again: with 16
+// places, the smallest key given up first, two sets of fields did not fit.)
+constexpr size_t kMaxGraphs = 64;
+template <class Step>
+int run_graph(igg_grid *g, const GraphKey &key, int n, Step step, cudaGraphExec_t *out) {
+  auto it = g->graphs.find(key);
+  if (it == g->graphs.end()) {
+    cudaError_t e = cudaStreamBeginCapture(g->cap, cudaStreamCaptureModeThreadLocal);
+    if (e != cudaSuccess) return cuda_error(e, "cudaStreamBeginCapture");
+    int rc = IGG_OK;
+    for (int k = 0; k < n && rc == IGG_OK; ++k) rc = step(k);
+    cudaGraph_t graph = nullptr;
+    e = cudaStreamEndCapture(g->cap, &graph);
+    if (rc != IGG_OK) {
+      if (graph) cudaGraphDestroy(graph);
+      return rc;
+    }
+    if (e != cudaSuccess) return cuda_error(e, "cudaStreamEndCapture");
+    cudaGraphExec_t exec = nullptr;
+    e = cudaGraphInstantiateWithFlags(&exec, graph, cudaGraphInstantiateFlagUseNodePriority);
+    cudaGraphDestroy(graph);
+    if (e != cudaSuccess) return cuda_error(e, "cudaGraphInstantiate");
+    if (g->graphs.size() >= kMaxGraphs) {
+      auto old = std::min_element(g->graphs.begin(), g->graphs.end(), [](auto &a, auto &b) {
+        return a.second.used < b.second.used;
+      });
+      cudaGraphExecDestroy(old->second.exec);
+      g->graphs.erase(old);
+    }
+    it = g->graphs.emplace(key, igg_grid::Graph{exec, 0}).first;
+  }
+  it->second.used = ++g->graph_uses;
+  *out = it->second.exec;
+  return IGG_OK;
+}
+
 int check_widths(const igg_grid *g, const int *w) {
   if (!w) return IGG_OK;
   for (int d = 0; d < 3; ++d) {
@@ -1037,7 +1081,7 @@ int check_widths(const igg_grid *g, const int *w) {
 
 void destroy_grid(igg_grid *g) {
   if (!g) return;
-  for (auto &kv : g->graphs) cudaGraphExecDestroy(kv.second);
+  for (auto &kv : g->graphs) cudaGraphExecDestroy(kv.second.exec);
   for (auto &kv : g->split) {
     for (auto &b : kv.second.boundary) free_tiles(b);
     free_tiles(kv.second.inner);
@@ -1434,7 +1478,9 @@ int igg_run(igg_grid *g, int nt, const int widths[3], void *T, void *T2, const v
   };
   // The steps [i0, i1) run as launches of a graph of two steps each, on small
   // grids, where a graph launch costs as much as a step, of up to 16 steps (one
-  // 64^3 FP64 array, 100 steps: 512 us with graphs of two, 326 us of fourteen).
+  // 64^3 FP64 array, 100 steps: 512 us with graphs of two, 326 us of fourteen;
+  // composed of fixed lengths of 16, 8, 4 and two steps, 14 steps took 67 instead
+  // of 59 us).
   //
   // Where the kernel can read a neighbour's points in place of halo cells
   // (virt_applies), only the last two steps update the halo (both buffers end
@@ -1482,30 +1528,9 @@ int igg_run(igg_grid *g, int nt, const int widths[3], void *T, void *T2, const v
                        widths ? widths[0] : 0, widths ? widths[1] : 0, widths ? widths[2] : 0, c.wx,
                        c.wy, c.wz, c.wc);
     cudaGraphExec_t exec = nullptr;
-    auto it = g->graphs.find(key);
-    if (it != g->graphs.end()) {
-      exec = it->second;
-    } else {
-      cudaError_t e = cudaStreamBeginCapture(g->cap, cudaStreamCaptureModeThreadLocal);
-      if (e != cudaSuccess) return cuda_error(e, "cudaStreamBeginCapture");
-      int rc = IGG_OK;
-      for (int k = 0; k < 2 * per && rc == IGG_OK; ++k) rc = step(i0 + k, mid, g->cap);
-      cudaGraph_t graph = nullptr;
-      e = cudaStreamEndCapture(g->cap, &graph);
-      if (rc != IGG_OK) {
-        if (graph) cudaGraphDestroy(graph);
-        return rc;
-      }
-      if (e != cudaSuccess) return cuda_error(e, "cudaStreamEndCapture");
-      e = cudaGraphInstantiateWithFlags(&exec, graph, cudaGraphInstantiateFlagUseNodePriority);
-      cudaGraphDestroy(graph);
-      if (e != cudaSuccess) return cuda_error(e, "cudaGraphInstantiate");
-      if (g->graphs.size() >= 16) {  // bounded cache
-        cudaGraphExecDestroy(g->graphs.begin()->second);
-        g->graphs.erase(g->graphs.begin());
-      }
-      g->graphs.emplace(key, exec);
-    }
+    if (int rc = run_graph(
+            g, key, 2 * per, [&](int k) { return step(i0 + k, mid, g->cap); }, &exec))
+      return rc;
     NvtxRange r("igg_run graph launches");
     for (; i + 2 * per <= i1; i += 2 * per) {
       cudaError_t e = cudaGraphLaunch(exec, s);
@@ -1799,7 +1824,7 @@ int igg_grid_set_option(igg_grid *g, int option, int value) {
   else if (option == IGG_OPT_HIDE_HALO) g->hide_halo = value != 0;
   else g->fused_halo = value != 0;
   // tile tables and graphs depend on the kernel choice
-  for (auto &kv : g->graphs) cudaGraphExecDestroy(kv.second);
+  for (auto &kv : g->graphs) cudaGraphExecDestroy(kv.second.exec);
   g->graphs.clear();
   for (auto &kv : g->split) {
     for (auto &b : kv.second.boundary) free_tiles(b);
