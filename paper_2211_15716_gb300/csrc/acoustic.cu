@@ -93,9 +93,8 @@ __device__ __forceinline__ void ac_ahead(const S *p) {
 
 template <class S>
 __global__ void __launch_bounds__(kAcX *kAcY)
-    k_acoustic_v(int nx, int ny, int nz, int zchunks, const S *P, S *__restrict__ Vx,
-                 S *__restrict__ Vy, S *__restrict__ Vz, const AcW<S> w,
-                 const int *__restrict__ nbr, int ox, int xsend, int ahead) {
+    k_acoustic_v(int nx, int ny, int nz, int zchunks, const S *P, S *Vx, S *Vy, S *Vz,
+                 const AcW<S> w, const int *__restrict__ nbr, int ox, int xsend, int ahead) {
   using N = AcNum<S>;
   const int i = blockIdx.x * kAcX + threadIdx.x, j = blockIdx.y * kAcY + threadIdx.y;
   if (i >= nx || j >= ny) return;
@@ -186,7 +185,7 @@ __global__ void __launch_bounds__(kAcX *kAcY)
 
 template <class S>
 __global__ void __launch_bounds__(kAcX *kAcY)
-    k_acoustic_p(int nx, int ny, int nz, int zchunks, S *__restrict__ P,
+    k_acoustic_p(int nx, int ny, int nz, int zchunks, S *P,
                  const S *Vx, const S *Vy, const S *Vz, const AcW<S> w,
                  const int *__restrict__ nbr, int ox, int xsend, int ahead) {
   using N = AcNum<S>;

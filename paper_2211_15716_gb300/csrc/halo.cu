@@ -17,7 +17,7 @@ namespace {
 // rows contiguous (sa = 1) and 16-byte aligned, copied as 16-byte vectors.
 template <class E, bool VEC>
 __global__ void __launch_bounds__(256)
-    k_halo_planes(const PlaneCopy *__restrict__ copies, E *__restrict__ f, int na, int nb,
+    k_halo_planes(const PlaneCopy *__restrict__ copies, E *f, int na, int nb,
                   long long sa, long long sb) {
   const int ci = blockIdx.x / nb, b = blockIdx.x % nb;
   const PlaneCopy c = copies[ci];
@@ -96,7 +96,7 @@ __device__ __forceinline__ void gather_step(const HaloGather &h, int d, int &s, 
 }
 
 template <class E, bool VEC>
-__global__ void __launch_bounds__(256) k_halo_gather(E *__restrict__ f, const HaloGather h) {
+__global__ void __launch_bounds__(256) k_halo_gather(E *f, const HaloGather h) {
   const int nx = h.n[0], ny = h.n[1], nz = h.n[2];
   const int rows = 2 * ny + (h.skipx ? 2 : 4) * (nz - 2);
   const int s0 = (int)(blockIdx.x / rows);
@@ -168,7 +168,7 @@ __global__ void __launch_bounds__(256) k_halo_gather(E *__restrict__ f, const Ha
 // 2o - 1 points, where o - 1 = n - o feeds both: the adds are atomic.
 template <class E>
 __global__ void __launch_bounds__(256)
-    k_halo_planes_adj(const PlaneCopy *__restrict__ copies, E *__restrict__ f, int na, int nb,
+    k_halo_planes_adj(const PlaneCopy *__restrict__ copies, E *f, int na, int nb,
                       long long sa, long long sb) {
   const int ci = blockIdx.x / nb, b = blockIdx.x % nb;
   const PlaneCopy c = copies[ci];

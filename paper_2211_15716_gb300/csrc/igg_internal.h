@@ -19,9 +19,10 @@ namespace igg {
 // writes visible); before it, a kernel may only set up its shared memory and
 // read tables that no launch writes. pdl_trigger() lets the next launch start
 // as soon as every block of this one is running. Data that earlier launches
-// write must not be read through the read-only path (__ldg, const __restrict__
-// pointers) in such a kernel: the compiler may move those loads above the
-// wait. A step of a small grid is a chain of launches a few microseconds long:
+// write must not be read through the read-only path (__ldg) or through any
+// __restrict__ pointer in such a kernel: the compiler may move those loads above
+// the wait, whose asm does not have the pointer among its operands. (Tables that
+// no launch writes, and memory that the kernel only stores to, may be restricted.) A step of a small grid is a chain of launches a few microseconds long:
 // one 64^3 FP64 array, 100 steps, 1.20 to 1.17 ms; FP32 misfit gradient on 2x2x2 x
 // 64^3, 32 steps, 2.49 to 1.95 ms. Launches over more points (pdl_on) go
 // without: there the early blocks of the next launch only take slots from the
