@@ -245,13 +245,14 @@ struct FixShared {
 static_assert(sizeof(FixShared) <= 8 * kFixPend * sizeof(FixEntry), "in the staging's place");
 
 // Tm, Tc, Tn, Cn: the T planes m - 1, m, m + 1 and the Ci plane; warp: the
-// consumer warp, whose rows are warp and warp + H / 2; d0: the first row's place
-// in T2, the second row dj elements further. def: bits 0, 1 the first row's two
+// consumer warp, whose rows are warp and warp + H / 2; p0: the first row's place
+// in T2 (of npts elements), the second row dj elements further. def: bits 0, 1 the first row's two
 // points of this lane, bits 2, 3 the second's.
 template <int NG, bool SWAP>
 __device__ __forceinline__ void emu_fix_rows(const double *Tm, const double *Tc, const double *Tn,
-                                             const double *Cn, int warp, double *d0, long long dj,
-                                             unsigned def, const W<double> &w, FixShared *fs) {
+                                             const double *Cn, int warp, double *T2, long long p0,
+                                             long long dj, long long npts, unsigned def,
+                                             const W<double> &w, FixShared *fs) {
   using Sh = TmaShape<double, 32, 16>;
   constexpr unsigned kAll = 0xffffffffu;
   const int lane = threadIdx.x & 31;
@@ -287,7 +288,8 @@ __device__ __forceinline__ void emu_fix_rows(const double *Tm, const double *Tc,
     bool ok;
     double v = cell_emu_aligned<NG>(*pc, nb, ci, w, ok);
     if (!ok) v = cell_f64(*pc, tn[0], tn[1], tn[2], tn[3], tn[4], tn[5], ci, w);
-    d0[(j ? dj : 0) + x] = v;
+    const long long p = p0 + (j ? dj : 0) + x;
+    if (in_bounds(p, npts)) T2[p] = v;
   }
   __syncwarp();  // the list before its next use
 }
@@ -652,8 +654,9 @@ __global__ void __launch_bounds__(32 * 9, INL ? 2 : IGG_TMA_MIN_BLOCKS)
       if constexpr (INL) {
         if (__any_sync(0xffffffffu, def != 0u))
           emu_fix_rows<emu_groups(MODE), SWAP>(
-              reinterpret_cast<const S *>(smem + (k - 1) % NS * Sh::STAGE), Tc, Tn, Cn, warp,
-              T2 + t.base + t.x0 + srow * (t.r0 + warp) + smarch * m, srow * (Sh::H / 2), def, w, fs);
+              reinterpret_cast<const S *>(smem + (k - 1) % NS * Sh::STAGE), Tc, Tn, Cn, warp, T2,
+              t.base + t.x0 + srow * (t.r0 + warp) + smarch * m, srow * (Sh::H / 2), c0.npts, def, w,
+              fs);
       }
       __syncwarp();
       // load k's stage (INL: load k - 1's) back to the producer

@@ -42,3 +42,18 @@ def test_no_restricted_reads_behind_the_dependency_wait():
         for p in restricted & STORED:  # (reads through the pointer itself)
             assert not re.search(r"=\s*\*?%s\s*\[" % p, body), (file, name, p)
         assert "__ldg" not in body, (file, name)
+
+
+def test_stores_of_the_stencils_are_bounds_checked():
+    """Every function of the stencil that stores to T2 tests its index in the
+    bounds-checked build."""
+    seen = 0
+    for file in ("tma.cu", "rows.cu"):
+        src = open(os.path.join(CSRC, file)).read()
+        for m in re.finditer(r"^(?:template <[^>]*>\n)?__(?:global|device)__[^;{]*?(\w+)\([^;{]*\{\n(.*?)^\}",
+                             src, re.M | re.S):
+            body = m.group(2)
+            if re.search(r"(T2|d0|dst)(\[[^\]]*\])+ = |\*reinterpret_cast<uint4 \*>\(dst\) =", body):
+                seen += 1
+                assert "in_bounds(" in body, (file, m.group(1))
+    assert seen >= 4  # k_stencil_tma, emu_fix_rows, k_fixup_f64, k_stencil_rows
