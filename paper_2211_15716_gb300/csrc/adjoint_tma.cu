@@ -8,8 +8,7 @@
 // of the work order (z chunk, column of a subdomain, plane), so every CTA
 // handles the same number of planes; a share splits into segments (runs of
 // planes of one column). All subdomains go in one launch: with a launch each,
-// eight subdomains of 64^3 left most of the GPU idle eight times over
-// (FP32
+// eight subdomains of 64^3 left most of the GPU idle eight times over (FP32
 // misfit gradient of 32 steps there: 4.72 to 2.49 ms).
 //
 // Per plane p, cp.async.bulk.tensor (TMA) loads into a ring of NS shared-
@@ -109,7 +108,6 @@ __global__ void __launch_bounds__(32 * AdjShape<S>::WARPS, AdjShape<S>::MINB)
   using Sh = AdjShape<S>;
   using Ops = AdjOps<S>;
   using VT = typename Sh::VT;
-  using LT = typename Ops::LT;
   constexpr int V = Sh::V, W = Sh::W, BW = Sh::BW, H = Sh::H, NS = Sh::NS;
   constexpr unsigned NT = 32 * Sh::WARPS;
   extern __shared__ __align__(128) unsigned char smem[];

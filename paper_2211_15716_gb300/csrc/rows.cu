@@ -128,16 +128,12 @@ __global__ void __launch_bounds__(32 * 9, 3)
       }
       if (__any_sync(0xffffffffu, flags[0] != 0)) break;
       const long long pT = t.base + sz * (t.m0 - 1 + k);
+      // (a tile has m0, r0, xb >= 1: eT >= 0)
       const long long eT = pT + (long long)nx * (t.r0 - 1 + lane) + t.xb - 1;
       const long long eC = pT - sz + (long long)nx * (t.r0 + lane) + t.xb;
-      long long aT = eT - (eT & (V - 1)), bT = (eT + (t.xe - t.xb) + 2 + V - 1) / V * V;
-      long long aC = eC - (eC & (V - 1)), bC = (eC + (t.xe - t.xb) + V - 1) / V * V;
-      // (eT >= -1; a copy that starts before the field starts at 0 instead)
-      int dT = 0;
-      if (aT < 0) {
-        aT = 0;
-        dT = V;
-      }
+      const long long aT = eT - (eT & (V - 1)), aC = eC - (eC & (V - 1));
+      long long bT = (eT + (t.xe - t.xb) + 2 + V - 1) / V * V;
+      long long bC = (eC + (t.xe - t.xb) + V - 1) / V * V;
       bT = min(bT, lim);
       bC = min(bC, lim);
       const unsigned nT = hasT && bT > aT ? (unsigned)(bT - aT) * 8u : 0u;
@@ -146,7 +142,7 @@ __global__ void __launch_bounds__(32 * 9, 3)
       const unsigned bar = full0 + 8 * s, dst = sbase + s * Sh::STAGE;
       if (lane == 0) mbar_expect_tx(bar, total);
       __syncwarp();
-      if (nT) bulk_row(dst + (unsigned)((lane * Sh::BW + dT) * 8), T + aT, nT, bar);
+      if (nT) bulk_row(dst + (unsigned)(lane * Sh::BW * 8), T + aT, nT, bar);
       if (nC)
         bulk_row(dst + Sh::TB + (unsigned)(lane * Sh::CW * 8), Ci + aC, nC, bar);
     }

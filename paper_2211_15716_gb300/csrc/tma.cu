@@ -248,7 +248,7 @@ static_assert(sizeof(FixShared) <= 8 * kFixPend * sizeof(FixEntry), "in the stag
 // consumer warp, whose rows are warp and warp + H / 2; p0: the first row's place
 // in T2 (of npts elements), the second row dj elements further. def: bits 0, 1 the first row's two
 // points of this lane, bits 2, 3 the second's.
-template <int NG, bool SWAP>
+template <int NG>
 __device__ __forceinline__ void emu_fix_rows(const double *Tm, const double *Tc, const double *Tn,
                                              const double *Cn, int warp, double *T2, long long p0,
                                              long long dj, long long npts, unsigned def,
@@ -279,9 +279,8 @@ __device__ __forceinline__ void emu_fix_rows(const double *Tm, const double *Tc,
     const int q = list[i], j = q >> 6, x = q & 63, r = warp + j * (Sh::H / 2);
     const int o = (r + 1) * Sh::BW + Sh::V + x;
     const double *pc = Tc + o;
-    const double up = pc[-Sh::BW], dn = pc[Sh::BW], m = Tm[o], n = Tn[o], ci = Cn[r * Sh::W + x];
-    const double tn[6] = {pc[-1],        pc[1],         SWAP ? m : up,
-                          SWAP ? n : dn, SWAP ? up : m, SWAP ? dn : n};
+    const double ci = Cn[r * Sh::W + x];
+    const double tn[6] = {pc[-1], pc[1], pc[-Sh::BW], pc[Sh::BW], Tm[o], Tn[o]};
     unsigned long long nb[6];
 #pragma unroll
     for (int k = 0; k < 6; ++k) nb[k] = dbits(tn[k]);
@@ -621,7 +620,8 @@ __global__ void __launch_bounds__(32 * 9, INL ? 2 : IGG_TMA_MIN_BLOCKS)
           }
         }
         if constexpr (INL) {
-          static_assert(is_emu(MODE) && LPR == 32 && V == 2 && Sh::RPT == 2, "two rows per warp");
+          static_assert(is_emu(MODE) && !SWAP && LPR == 32 && V == 2 && Sh::RPT == 2,
+                        "two rows along y per warp");
           if (comp[j]) def |= (~okm & inm) << (2 * j);
         } else if constexpr (is_emu(MODE)) {
           // The warp owns the whole row (one row per warp, two points per
@@ -653,7 +653,7 @@ __global__ void __launch_bounds__(32 * 9, INL ? 2 : IGG_TMA_MIN_BLOCKS)
       }
       if constexpr (INL) {
         if (__any_sync(0xffffffffu, def != 0u))
-          emu_fix_rows<emu_groups(MODE), SWAP>(
+          emu_fix_rows<emu_groups(MODE)>(
               reinterpret_cast<const S *>(smem + (k - 1) % NS * Sh::STAGE), Tc, Tn, Cn, warp, T2,
               t.base + t.x0 + srow * (t.r0 + warp) + smarch * m, srow * (Sh::H / 2), c0.npts, def, w,
               fs);
