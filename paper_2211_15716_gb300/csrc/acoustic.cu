@@ -262,8 +262,9 @@ cudaError_t launch_t(int nsub, int nx, int ny, int nz, void *P, void *Vx, void *
   // room on, and where those are neither idle nor soon drained the FP64 pipes end
   // up with unequal shares (16 steps, early start against none: 64^3, 32 CTAs,
   // 547 and 610 us; 2x1x2 x 70x60x64, 192, 1762 and 1022; 2x1x1 x 128^3, 512,
-  // 2137 and 2023; 2x1x2 x 200x160x128, 2240, 6492 and 6590). FP32 launches gain
-  // at every size.
+  // 2137 and 2023; 2x1x2 x 200x160x128, 2240, 6492 and 6590). So up to one CTA per
+  // SM (152 SMs), and again above eight; where between 512 and 2240 CTAs the
+  // upper line lies was not measured. FP32 launches gain at every size.
   const long long ctas = (long long)grid.x * grid.y * grid.z;
   const bool pdl = sizeof(S) == 4 || ctas <= 152 || ctas > 2 * 4 * 152;
   // (kAcAhead: fields that stay in L2 only lose issue slots to the prefetches)

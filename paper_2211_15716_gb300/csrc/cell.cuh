@@ -511,10 +511,9 @@ __device__ __forceinline__ double cell_emu_fast(double tc, const unsigned long l
 // shifted value (0 and subnormals, whose leading bit is not there, are shifted
 // out: er >= 180 where the path applies), and (h + 1) >> 1 rounds to the nearest,
 // halves away from zero for either sign. Seven of these are most of the fix-up
-// launch's work, which the integer pipe bounds (73 % busy): with a masked
-// significand, a conditional rounding shift and a conditional negation (about 24
-// instructions instead of 17) twenty steps of the field above took 10.43 instead
-// of 9.86 ms.
+// launch's work, which the integer pipe bounds: with a masked significand, a
+// conditional rounding shift and a conditional negation (about 24 instructions
+// instead of 17) twenty steps of the field above took 12.74 instead of 11.87 ms.
 __device__ __forceinline__ unsigned long long emu3_aligned(unsigned long long b, unsigned hc,
                                                            unsigned er10) {
   const unsigned hi = (unsigned)(b >> 32);

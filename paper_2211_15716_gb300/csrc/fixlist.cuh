@@ -17,8 +17,8 @@ struct FixEntry {
 // Entries a consumer warp stages in shared memory before it reserves their
 // slots in the list with one atomic (a warp waits for each atomic's return:
 // with 16 entries twenty steps of 2x2x2 x 256x128x128, modes up to 8 about 0,
-// took 8.61 ms, with 32, as many as one store of the warp appends, 8.59; ten steps
-// of 2x2x2 x 512x256x256, smooth, 10.38 and 10.37).
+// took 11.91 ms, with 32, as many as one store of the warp appends, 11.87; ten
+// steps of 2x2x2 x 512x256x256, smooth, 10.35 and 10.33).
 constexpr unsigned kFixPend = 32;
 struct FixList {
   FixEntry *e;

@@ -271,11 +271,11 @@ struct GpShape {
   static constexpr int V = 16 / (int)sizeof(S);          // points per lane
   static constexpr int W = 32 * V;                       // points per row
   static constexpr int BW = W + 2 * V;                   // w box width
-  // rows per tile and stages: FP64 8 and 4, three CTAs per SM; FP32 16 and 6, one.
-  // The FP64 launch is bound by instruction issue (255 instructions per point,
-  // 2.4 per clock at 15 warps per SM, the barrier of each plane its first
-  // stall): 2x2x2 x 256^3, four steps, with one CTA of 16 rows 10.79, two of 8
-  // (six stages) 11.29, three of 8 10.76 ms
+  // rows per tile and stages: FP64 8 and 4, three CTAs per SM (24 warps); FP32 16
+  // and 6, one. The FP64 launch is bound by instruction issue (263 instructions
+  // per point, issue 66 %), then by the barrier of each plane; the shape matters
+  // little: 2x2x2 x 256^3, four steps, three CTAs of 8 rows 10.76, one of 16 rows
+  // 10.79, two of 8 (six stages) 11.29 ms
   static constexpr int H = sizeof(S) == 8 ? 8 : 16;
   static constexpr int BH = H + 2;
   static constexpr int WARPS = H;

@@ -93,10 +93,11 @@ template <class S>
 __device__ __forceinline__ void lds_vec(const S *p, Vec<S> &o) {
   unpack(*reinterpret_cast<const uint4 *>(p), o);
 }
-// Fix-up blocks: one wave, five per SM (48 registers). Against 8 x 152, ten steps
-// of 2x2x2 x 512x256x256 10.37 and 10.33 ms, of 2x2x2 x 255x127x129 1.857 and
-// 1.814, 48 steps of the misfit gradient at 256^3 20.60 and 20.23, many points
-// listed (k_fixup_f64's field) 8.56 both; 4 x 152: 8.74 there, the others equal.
+// Fix-up blocks: one wave, five per SM (48 registers) of 152 SMs. Against 8 x 152,
+// ten steps of 2x2x2 x 512x256x256 10.36 and 10.33 ms, of 2x2x2 x 255x127x129 1.854
+// and 1.813, 48 steps of the misfit gradient at 256^3 20.73 and 20.27; with many
+// points listed (k_fixup_f64's field) 11.43 and 11.87. 4 x 152: 12.12 there, the
+// others equal.
 constexpr int kFixupBlocks = 5 * 152;
 
 // bit i of x (i < 16) to bit 2i
@@ -699,12 +700,12 @@ __global__ void __launch_bounds__(32 * 9, INL ? 2 : IGG_TMA_MIN_BLOCKS)
 // them are there: its eight FP64 instructions hold the SM's FP64 pipe for 128
 // cycles however few lanes need them.
 // The integer work of the aligned path bounds the launch where many points are
-// listed (2x2x2 x 256x128x128, modes up to 8 about 0: half of them), the latency
-// of its loads where few are. Twenty steps of that field: points dealt to the
-// lanes from batches of four entries by their rank, or a lane per point of the
-// segment for entries of 16 and more, 9.86 ms; with the list 8.59. (Batches of 4
-// and 16 entries 8.56 and 8.66; ten steps of 2x2x2 x 512x256x256, smooth, 10.40
-// before, 10.37 with 8, 10.38 with 4 and 16.)
+// listed (2x2x2 x 256x128x128, modes up to 8 about 0: 84 %), the latency
+// of its loads where few are. With 8 x 152 blocks, points dealt to the lanes from
+// batches of four entries by their rank, or a lane per point of the segment for
+// entries of 16 and more: twenty steps of that field 11.74 ms, with the list 11.43.
+// (Batches of 4 and 16 entries 11.90 where 8 take 11.87; ten steps of 2x2x2 x
+// 512x256x256, smooth, 10.32 and 10.33 where 8 take 10.33.)
 // Each block adds its segments and points to the list's totals; the last
 // block to finish resets the list.
 constexpr unsigned kFixBatch = 8;
