@@ -183,7 +183,8 @@ int igg_selftest_bounded_wait(unsigned *status);
  *     TMA-pipelined kernel when the row length is a multiple of 16 bytes; 0
  *     selects the register-pipelined vector kernel. Bit-identical results.
  *   IGG_OPT_F64_EMU (default 1): F64 fields use the emulated FP64 cell: for
- *     points whose 7 stencil values share sign and exponent, the second
+ *     points whose 7 stencil values share sign and exponent (and whose second
+ *     differences stay below 2^45 of their ulps), the second
  *     differences are formed exactly from the bit patterns as integers,
  *     weighted in float-float pairs and applied with one FP64 FMA and an
  *     integer ulp correction (per-step error within about one ulp of T2 plus
@@ -194,9 +195,9 @@ int igg_selftest_bounded_wait(unsigned *status);
  *     overflow or underflow, weights above 2^40) use the FP64 cell (8 FP64
  *     instructions per point). On the TMA kernel the points outside the
  *     one-FMA path go to a fix-up launch, so fields where many stencils
- *     change sign or exponent step about three times slower (a field that
- *     changes sign: 3.0 x the time of a smooth one, below the FP64
- *     cell's 3.6 x; see igg_fixup_stats).
+ *     change sign or exponent step several times slower (a field that changes
+ *     sign: 2.6 x the time of a smooth one, a field of short waves 4.6 x, the
+ *     FP64 cell 4.0 x; see igg_fixup_stats).
  *   IGG_OPT_FUSED_HALO (default 1): igg_step_hidden (and igg_run with
  *     widths) run as the full step launch followed by the one-launch halo
  *     update (all subdomains being in the device's memory, no transfer is
